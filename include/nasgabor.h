@@ -502,9 +502,13 @@ size_t nasg_raster_workspace_bytes(int64_t n, int32_t width, int32_t height, int
  *          output (transmittance left at each pixel).
  *   workspace: device, 256-byte aligned, >= nasg_raster_workspace_bytes(n, w, h,
  *          max_pairs); it keeps the forward's state for nasg_raster_backward.
- *   n_pairs: nullable host output, the number of (tile, primitive) pairs.
- * Synchronises the stream once (to size the sort). NASG_ERR_CAPACITY when the
- * pairs exceed max_pairs (n_pairs still reports the count); n < 2^31.
+ *   n_pairs: nullable host output, the number of (tile, primitive) pairs of the
+ *          primitives' footprint squares (the lists hold those whose ellipse reaches
+ *          the tile, a part of them).
+ * The host waits once, for the projection (to size the sort). NASG_ERR_CAPACITY when
+ * the pairs exceed max_pairs (n_pairs still reports the count); n < 2^31. The lists'
+ * device-side waits are bounded: should one give up, nasg_device_status() says so and
+ * the image is empty.
  */
 nasg_status nasg_raster_forward(int64_t n, const float* means, const float* scales, const float* quats,
                                 const float* opacity, const float* colours, const nasg_raster_camera* camera,

@@ -59,4 +59,58 @@ NASG_COVER_HD bool cover_box(float A, float B2, float C, CoverSlopes r, float li
   return !(q1 > limit && q2 > limit);
 }
 
+// The same ellipse by tile rows: for a row of tiles, the tiles whose pixel centres the ellipse
+// q <= limit can reach. With dy held, the ellipse spans u + r dy -+ sqrt(h (limit - dy^2 / sc)),
+// r = sb / sc, h = det / sc; over a band of dy its right end is furthest at dy = y_right =
+// sb sqrt(limit / sa) or, that outside the band, at the band's nearer end (the right boundary is
+// concave in dy), its left end at -y_right likewise. The launches that count and that list the
+// tiles must agree, so on the device every operation is one that the compiler cannot contract.
+struct CoverRows {
+  float u, v, r, h;
+  float limit, isc, y_right, unused;
+};
+
+#if defined(__CUDA_ARCH__)
+__device__ __forceinline__ float cover_sqrt(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+#define NASG_COVER_MUL __fmul_rn
+#define NASG_COVER_ADD __fadd_rn
+#define NASG_COVER_FMA __fmaf_rn
+#define NASG_COVER_SQRT cover_sqrt
+#else
+#define NASG_COVER_MUL(a, b) ((a) * (b))
+#define NASG_COVER_ADD(a, b) ((a) + (b))
+#define NASG_COVER_FMA(a, b, c) fmaf(a, b, c)
+#define NASG_COVER_SQRT sqrtf
+#endif
+
+NASG_COVER_HD CoverRows cover_rows(float u, float v, float sa, float sb, float sc, float det, float limit) {
+  const float isc = 1.f / sc;
+  return {u, v, sb * isc, det * isc, limit, isc, sb * sqrtf(limit / sa), 0.f};
+}
+
+// Tiles [*c0, *c1] of tile row `row` (16 x 16 tiles), within [x0, x1]; false for none. The 0.05 px
+// cover the rounding of means within 32768 pixels.
+NASG_COVER_HD bool cover_row(const CoverRows& c, int row, int x0, int x1, int* c0, int* c1) {
+  *c0 = x0;
+  *c1 = x1;
+  if (!(c.limit < INFINITY)) return true;
+  const float yl = NASG_COVER_ADD(float(16 * row) + 0.5f, -c.v), yh = NASG_COVER_ADD(float(16 * row) + 15.5f, -c.v);
+  const float yr = fminf(fmaxf(c.y_right, yl), yh), ye = fminf(fmaxf(-c.y_right, yl), yh);
+  const float tr = NASG_COVER_FMA(NASG_COVER_MUL(-yr, yr), c.isc, c.limit);
+  const float te = NASG_COVER_FMA(NASG_COVER_MUL(-ye, ye), c.isc, c.limit);
+  if (tr < 0.f && te < 0.f) return false;
+  const float right = NASG_COVER_ADD(NASG_COVER_FMA(c.r, yr, c.u), NASG_COVER_SQRT(NASG_COVER_MUL(c.h, fmaxf(tr, 0.f))));
+  const float left = NASG_COVER_ADD(NASG_COVER_FMA(c.r, ye, c.u), -NASG_COVER_SQRT(NASG_COVER_MUL(c.h, fmaxf(te, 0.f))));
+  // tile t holds the centres 16 t + 0.5 .. 16 t + 15.5
+  const float lo = ceilf(NASG_COVER_MUL(NASG_COVER_ADD(left, -15.55f), 0.0625f));
+  const float hi = floorf(NASG_COVER_MUL(NASG_COVER_ADD(right, -0.45f), 0.0625f));
+  *c0 = int(fminf(fmaxf(lo, float(x0)), float(x1 + 1)));
+  *c1 = int(fmaxf(fminf(hi, float(x1)), float(x0 - 1)));
+  return *c0 <= *c1;
+}
+
 }  // namespace nasg

@@ -58,3 +58,47 @@ def test_window_matches_oracle(lib, w, h, win, n, log_scale):
     assert np.abs(rc).max() > 0
     assert rel_l2(gc.cpu().numpy(), rc) <= 1e-4
     assert rel_l2(go.cpu().numpy(), ro) <= 1e-4
+
+
+# The binning at the edges of its forms: one tile, 256 tiles (a single-digit tile key), keys of three
+# and four digits (over 256 tile columns or rows), lists shorter and longer than a sort block of
+# either shape, primitives that span more tiles than a thread lists alone, depths that tie by the
+# hundred (order by index), nothing but ties, and more primitives than the small depth blocks take.
+@pytest.mark.parametrize("w,h,n,log_scale,depths", [
+    (16, 16, 40, (-3.0, -1.5), 0),
+    (256, 256, 900, (-3.5, -1.0), 3),
+    (4200, 40, 1100, (-4.0, -0.5), 0),
+    (24, 4200, 1100, (-4.0, -0.5), 5),
+    (4500, 4300, 700, (-3.5, -0.3), 2),
+    (640, 360, 4096, (-4.5, -2.5), 1),
+    (1280, 720, 20_000, (-4.5, -2.0), 40),
+    (640, 360, 450_000, (-6.5, -4.0), 1000),
+])
+def test_binning_forms(lib, w, h, n, log_scale, depths):
+    import torch
+    rng = np.random.default_rng(w + h + n)
+    half = np.array([1.0, 1.0 * h / w]) if w >= h else np.array([1.0 * w / h, 1.0])
+    means = np.concatenate([rng.uniform(-1.1, 1.1, (n, 2)) * half, rng.uniform(-1, 1, (n, 1))], axis=1)
+    if depths:
+        means[:, 2] = rng.integers(0, depths, n) * (1.0 / depths) - 0.5
+    sc = [means, np.exp(rng.uniform(*log_scale, (n, 3))) * half.min() ** 0.5, rng.normal(size=(n, 4)),
+          rng.uniform(0.01, 0.9, n), rng.uniform(0, 1, (n, 3))]
+    sc = [x.astype(np.float32) for x in sc]
+    fx = np.float32(max(w, h) / 0.5)
+    centre = (0.0, 0.0, -4.0)
+    cam = lib.raster_camera(np.eye(3), centre, w, h, fx)
+    r = lib.Raster(n, cam, 1 << 26)
+    img, T = r.forward(*[_dev(x) for x in sc])
+    lib.nasg_device_status()
+    pix = np.stack([rng.integers(0, w, 60), rng.integers(0, h, 60)], axis=1)
+    ocam = {"rot": np.eye(3), "centre": np.asarray(centre), "fx": fx, "fy": fx, "cx": 0.5 * w, "cy": 0.5 * h,
+            "near": np.float32(0.2)}
+    ref, tref, margin = orr.render(*sc, ocam, w, h, pixels=pix, with_margin=True)
+    ok = margin > MARGIN
+    assert ok.mean() > 0.7, ok.mean()
+    assert (tref < 1).any()
+    assert np.abs(img.cpu().numpy()[pix[:, 1], pix[:, 0]] - ref)[ok].max() <= 1e-4
+    assert np.abs(T.cpu().numpy()[pix[:, 1], pix[:, 0]] - tref)[ok].max() <= 1e-4
+    # lists that differ in order would differ in the image; a second run gives the same bits
+    again, _ = r.forward(*[_dev(x) for x in sc])
+    torch.testing.assert_close(again, img, rtol=0, atol=0)

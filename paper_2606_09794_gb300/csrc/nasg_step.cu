@@ -56,7 +56,14 @@ __device__ __forceinline__ uint16_t bf16_bits(float x) { return __bfloat16_as_us
 __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gsrc) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(smem_dst)), "l"(gsrc) : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// 16 bytes, past L1 (16-byte aligned addresses).
+__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(smem_dst)), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// Waits until at most N of the thread's committed groups are in flight.
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // One bias-corrected Adam update: m <- b1 m + (1-b1) g, v <- b2 v + (1-b2) g^2,
 // th <- th - (lr/bc1) m / (sqrt(v)/sqrt(bc2) + eps).
@@ -240,15 +247,57 @@ __device__ __forceinline__ void step_phase2(const StepArgs& s, IDX i, int l0, co
   }
 }
 
-// Shared memory of the step kernel: per thread, P gradient pairs and (EVEN) the
-// P master, m and v pairs of its two lobes, each plane-major over the block's
-// 256 threads (no sharing between threads, no barrier).
-template <int P, bool EVEN>
-constexpr size_t step_smem_bytes() { return size_t(EVEN ? 4 : 1) * P * 256 * sizeof(float2); }
+// How a step kernel moves master, m and v. kScalar: element loads in phase two (odd L, unaligned
+// buffers). kPairs: each lane copies its own lobe pairs to shared memory (8 bytes, through L1).
+// kQuads: neighbouring lanes share their copies, 16 bytes each, past L1 (L a multiple of
+// four, 16-byte aligned planes).
+enum StepMove { kScalar, kPairs, kQuads };
 
-template <int FRAME, typename IDX, bool EVEN, bool LOSS>
+// Shared memory of the step kernel: per thread, P gradient pairs and, but for kScalar, the P
+// master, m and v pairs of its two lobes, each plane-major over the block's 256 threads (kQuads
+// shares them between the two lanes of a quad, the others with no one).
+template <int P, int MOVE>
+constexpr size_t step_smem_bytes() {
+  return size_t(MOVE == kScalar ? 1 : 4) * P * 256 * sizeof(float2);
+}
+
+// The primitive of lane item t: its index, or none where t is past the end or the list's entry is
+// outside [0, N).
+template <typename IDX>
+__device__ __forceinline__ bool step_prim(const EvalArgs& a, IDX total, IDX t, IDX& i) {
+  if (t >= total) return false;
+  i = t >> a.slice_log2;
+  if (a.idx) {
+    const int32_t v = __ldg(a.idx + i);
+    if (v < 0) return false;
+    i = IDX(v);
+  }
+  return i < IDX(a.n);
+}
+
+// Copies the P planes of two neighbouring lanes' four lobes, the even lane those of even planes,
+// the odd lane the others. `slot`: the block's array; off: first of the four lobes in plane 0.
+template <int P, typename IDX>
+__device__ __forceinline__ void copy_quads(float2* slot, const float* planes, IDX off, IDX NL) {
+  const int odd = threadIdx.x & 1;
+  float2* dst = slot + (threadIdx.x & ~1u) + odd * 256;
+  off += IDX(odd) * NL;
+#pragma unroll
+  for (int p = 0; p < P; p += 2, off += 2 * NL)
+    if (p + 1 < P || !odd) cp_async16(dst + p * 256, planes + off);
+}
+
+// Bound: HBM, and how many bytes the SM has in flight (16 warps, 128 registers, issue 31 %). Copies
+// of 8 bytes land through L1, whose lines are what is left of 80 KB x 2 of shared memory: with
+// 100 KB per block (a master copy one item ahead) the step took 1.4 times as long. 16-byte copies
+// past L1 have no such limit and are half as many: 6e6-primitive shell, 45 % visible, 8 lobes,
+// 1102 -> 1024 us per camera (5.8 TB/s); every primitive 2221 -> 2034 us (6.5 TB/s). On top of them
+// a master copy (1043 us) or the list's entry (1053 us) one item ahead, or streaming stores of m
+// and v (1082 us), gained nothing.
+template <int FRAME, typename IDX, int MOVE, bool LOSS>
 __global__ void __launch_bounds__(256, 2) step_kernel(const StepArgs s) {
   constexpr int P = FrameTraits<FRAME>::P;
+  constexpr bool EVEN = MOVE != kScalar;
   extern __shared__ __align__(16) float2 step_smem[];
   const EvalArgs& a = s.e;
   int64_t items = a.n_items;
@@ -260,38 +309,81 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepArgs s) {
   const IDX total = IDX(items) << a.slice_log2;
   const IDX stride = IDX(gridDim.x) * blockDim.x;
   const float gscale = LOSS && items > 0 ? 2.f / (3.f * float(items)) : 0.f;  // d mean / d colour
+  constexpr int kSlots = P * 256;
   float2* gslot = step_smem + threadIdx.x;
-  float2* tslot = gslot + P * 256;
-  float2* mslot = tslot + P * 256;
-  float2* vslot = mslot + P * 256;
   const IDX L = IDX(a.n_lobes);
   const IDX NL = IDX(a.n) * L;
   const float* master = static_cast<const float*>(a.params);
-  // block-uniform loop: every lane of a warp reaches the shuffles in phase one
-  for (IDX t0 = IDX(blockIdx.x) * blockDim.x; t0 < total; t0 += stride) {
-    RawItem<float, P> cur;
-    IDX i = 0;
-    fetch_item<float, P, IDX, EVEN, true, true>(a, total, t0 + threadIdx.x, l0, cur, i);
-    if (EVEN && cur.ok && IDX(l0) < L) {
-      IDX off = i * L + IDX(l0);
+  if constexpr (MOVE == kQuads) {
+    float2* marr = step_smem + kSlots;
+    float2* varr = marr + kSlots;
+    float2* tarr = varr + kSlots;
+    const IDX lq = IDX(l0 & ~3);  // the quad's first lobe
+    const bool has_lobes = IDX(l0) < L;
+    // block-uniform loop: every lane of a warp reaches the shuffles in phase one
+    for (IDX t0 = IDX(blockIdx.x) * blockDim.x; t0 < total; t0 += stride) {
+      RawItem<float, P> cur;
+      IDX i = 0;
+      const bool ok = step_prim(a, total, t0 + threadIdx.x, i);
+      cur.ok = ok;
+      __syncwarp();  // the warp has read its slots
+      if (ok && has_lobes) copy_quads<P>(tarr, master, i * L + lq, NL);
+      cp_async_commit();
+      if (ok) {
+        if (has_lobes) {
+          copy_quads<P>(marr, s.m, i * L + lq, NL);
+          copy_quads<P>(varr, s.v, i * L + lq, NL);
+        }
 #pragma unroll
-      for (int p = 0; p < P; ++p, off += NL) {
-        cp_async8(tslot + p * 256, master + off);
-        cp_async8(mslot + p * 256, s.m + off);
-        cp_async8(vslot + p * 256, s.v + off);
+        for (int c = 0; c < 3; ++c) {
+          cur.mu[c] = __ldg(a.means + 3 * i + c);
+          cur.gc[c] = __ldg(a.g_rgb + 3 * i + c);
+          cur.c0[c] = __ldg(static_cast<const float*>(a.c0) + IDX(c) * IDX(a.n) + i);
+        }
       }
+      cp_async_commit();
+      cp_async_wait<1>();  // master has landed; m and v land during the arithmetic
+      __syncwarp();
+      if (ok && has_lobes) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) cur.w[p] = tarr[p * 256 + threadIdx.x];
+      }
+      const bool mine = step_phase1<FRAME, IDX, EVEN, LOSS>(s, cur, i, l0, gscale, gslot);
+      cp_async_wait<0>();
+      __syncwarp();
+      if (mine)
+        step_phase2<P, IDX, EVEN>(s, i, l0, gslot, tarr + threadIdx.x, marr + threadIdx.x, varr + threadIdx.x);
     }
-    const bool mine = step_phase1<FRAME, IDX, EVEN, LOSS>(s, cur, i, l0, gscale, gslot);
-    if (EVEN) cp_async_wait_all();
-    if (mine) step_phase2<P, IDX, EVEN>(s, i, l0, gslot, tslot, mslot, vslot);
+  } else {
+    float2* tslot = gslot + kSlots;
+    float2* mslot = tslot + kSlots;
+    float2* vslot = mslot + kSlots;
+    for (IDX t0 = IDX(blockIdx.x) * blockDim.x; t0 < total; t0 += stride) {
+      RawItem<float, P> cur;
+      IDX i = 0;
+      fetch_item<float, P, IDX, EVEN, true, true>(a, total, t0 + threadIdx.x, l0, cur, i);
+      if (EVEN && cur.ok && IDX(l0) < L) {
+        IDX off = i * L + IDX(l0);
+#pragma unroll
+        for (int p = 0; p < P; ++p, off += NL) {
+          cp_async8(tslot + p * 256, master + off);
+          cp_async8(mslot + p * 256, s.m + off);
+          cp_async8(vslot + p * 256, s.v + off);
+        }
+        cp_async_commit();
+      }
+      const bool mine = step_phase1<FRAME, IDX, EVEN, LOSS>(s, cur, i, l0, gscale, gslot);
+      if (EVEN) cp_async_wait<0>();
+      if (mine) step_phase2<P, IDX, EVEN>(s, i, l0, gslot, tslot, mslot, vslot);
+    }
   }
 }
 
-template <int FRAME, typename IDX, bool EVEN, bool LOSS>
+template <int FRAME, typename IDX, int MOVE, bool LOSS>
 static nasg_status launch_step_k(const StepArgs& s, cudaStream_t st) {
   constexpr int P = FrameTraits<FRAME>::P;
-  constexpr size_t smem = step_smem_bytes<P, EVEN>();
-  auto k = step_kernel<FRAME, IDX, EVEN, LOSS>;
+  constexpr size_t smem = step_smem_bytes<P, MOVE>();
+  auto k = step_kernel<FRAME, IDX, MOVE, LOSS>;
   if (const nasg_status e = ensure_smem_limit(reinterpret_cast<const void*>(k), smem); e != NASG_OK) return e;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
@@ -302,10 +394,18 @@ static nasg_status launch_step_k(const StepArgs& s, cudaStream_t st) {
   return check_launch();
 }
 
+template <int FRAME, typename IDX, bool LOSS>
+static nasg_status launch_step_move(const StepArgs& s, StepMove move, cudaStream_t st) {
+  switch (move) {
+    case kQuads: return launch_step_k<FRAME, IDX, kQuads, LOSS>(s, st);
+    case kPairs: return launch_step_k<FRAME, IDX, kPairs, LOSS>(s, st);
+    default: return launch_step_k<FRAME, IDX, kScalar, LOSS>(s, st);
+  }
+}
+
 template <int FRAME, typename IDX>
-static nasg_status launch_step_idx(const StepArgs& s, bool even, bool loss, cudaStream_t st) {
-  if (loss) return even ? launch_step_k<FRAME, IDX, true, true>(s, st) : launch_step_k<FRAME, IDX, false, true>(s, st);
-  return even ? launch_step_k<FRAME, IDX, true, false>(s, st) : launch_step_k<FRAME, IDX, false, false>(s, st);
+static nasg_status launch_step_idx(const StepArgs& s, StepMove move, bool loss, cudaStream_t st) {
+  return loss ? launch_step_move<FRAME, IDX, true>(s, move, st) : launch_step_move<FRAME, IDX, false>(s, move, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -512,17 +612,19 @@ extern "C" nasg_status nasgabor_fused_step(const nasg_desc* desc, const nasg_tra
   const bool even = desc->n_lobes % 2 == 0 && aligned(st->master, 8) && aligned(st->m, 8) && aligned(st->v, 8) &&
                     (!st->params_bf16 || aligned(st->params_bf16, 4));
   const int64_t NL = desc->n * desc->n_lobes;
+  const bool quads = even && desc->n_lobes % 4 == 0 && aligned(st->master, 16) && aligned(st->m, 16) && aligned(st->v, 16);
+  const StepMove move = quads ? kQuads : (even ? kPairs : kScalar);
   const int64_t lim = int64_t(1) << 31;
   const bool idx32 = NL * nasg_lobe_planes(desc->frame_mode) < lim && 3 * desc->n < lim &&
                      2 * (a.n_items << a.slice_log2) + (int64_t(1) << 24) < lim;
   cudaStream_t cs = as_stream(stream);
   const bool loss = loss_mode == NASG_LOSS_MSE;
   if (desc->frame_mode == NASG_FRAME_QUAT) {
-    return idx32 ? launch_step_idx<NASG_FRAME_QUAT, uint32_t>(s, even, loss, cs)
-                 : launch_step_idx<NASG_FRAME_QUAT, uint64_t>(s, even, loss, cs);
+    return idx32 ? launch_step_idx<NASG_FRAME_QUAT, uint32_t>(s, move, loss, cs)
+                 : launch_step_idx<NASG_FRAME_QUAT, uint64_t>(s, move, loss, cs);
   }
-  return idx32 ? launch_step_idx<NASG_FRAME_COS, uint32_t>(s, even, loss, cs)
-               : launch_step_idx<NASG_FRAME_COS, uint64_t>(s, even, loss, cs);
+  return idx32 ? launch_step_idx<NASG_FRAME_COS, uint32_t>(s, move, loss, cs)
+               : launch_step_idx<NASG_FRAME_COS, uint64_t>(s, move, loss, cs);
 }
 
 // ---------------------------------------------------------------------------

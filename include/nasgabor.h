@@ -255,7 +255,7 @@ size_t nasg_frustum_workspace_bytes(int64_t n);
  *   idx      device [n] int32 output, ascending primitive indices of the visible set
  *   n_visible device int32 output (the list length)
  *   workspace device scratch of nasg_frustum_workspace_bytes(n) bytes, 16-byte aligned
- * Deterministic. n < 2^31. Three kernel launches on `stream`, no host synchronisation.
+ * Deterministic. n < 2^31. Two kernel launches on `stream`, no host synchronisation.
  */
 nasg_status nasg_frustum_compact(int64_t n, const float* means, const float* rot, const float* center,
                                  float tan_half_fov, float near_z, int32_t* idx, int32_t* n_visible,

@@ -18,9 +18,9 @@
 // slice of lanes covers a primitive.
 //
 // Compaction: an ordered (deterministic, ascending) list of the primitives
-// whose centre is inside a pinhole frustum, in three launches: per-chunk
-// counts (and a visibility byte per primitive), one-block exclusive scan of the
-// counts (also the total), and the ordered scatter.
+// whose centre is inside a pinhole frustum, in two launches: per-block
+// counts (and a visibility bit per primitive), and the ordered scatter, whose
+// blocks sum the counts before theirs (the last one the total).
 #include <cmath>
 #include <mutex>
 
@@ -413,7 +413,8 @@ static nasg_status launch_step_idx(const StepArgs& s, StepMove move, bool loss, 
 // ---------------------------------------------------------------------------
 
 constexpr int kCompactBlock = 256;
-constexpr int kCompactChunk = 4096;  // primitives per block (16 rounds of 256)
+constexpr int kCompactChunk = 4096;      // primitives per round of a block (16 per thread)
+constexpr int kCompactMaxBlocks = 2048;  // a block sums the counts of all before it
 
 struct FrustumArgs {
   const float* means;
@@ -426,10 +427,10 @@ struct FrustumArgs {
 
 // Visibility of one centre with explicitly rounded operations, so that every
 // launch makes the identical decision.
-__device__ __forceinline__ bool in_frustum(const FrustumArgs& f, int64_t i) {
-  const float x = __fsub_rn(f.means[3 * i + 0], f.c[0]);
-  const float y = __fsub_rn(f.means[3 * i + 1], f.c[1]);
-  const float z = __fsub_rn(f.means[3 * i + 2], f.c[2]);
+__device__ __forceinline__ bool in_frustum(const FrustumArgs& f, float mx, float my, float mz) {
+  const float x = __fsub_rn(mx, f.c[0]);
+  const float y = __fsub_rn(my, f.c[1]);
+  const float z = __fsub_rn(mz, f.c[2]);
   const float px = __fmaf_rn(f.r[0], x, __fmaf_rn(f.r[1], y, __fmul_rn(f.r[2], z)));
   const float py = __fmaf_rn(f.r[3], x, __fmaf_rn(f.r[4], y, __fmul_rn(f.r[5], z)));
   const float pz = __fmaf_rn(f.r[6], x, __fmaf_rn(f.r[7], y, __fmul_rn(f.r[8], z)));
@@ -437,73 +438,139 @@ __device__ __forceinline__ bool in_frustum(const FrustumArgs& f, int64_t i) {
   return pz > f.near_z && fabsf(px) <= lim && fabsf(py) <= lim;
 }
 
-__global__ void __launch_bounds__(kCompactBlock) frustum_count_kernel(FrustumArgs f, uint8_t* flags,
-                                                                      int32_t* counts) {
-  const int64_t base = int64_t(blockIdx.x) * kCompactChunk;
-  int local = 0;
-  for (int r = 0; r < kCompactChunk / kCompactBlock; ++r) {
-    const int64_t i = base + r * kCompactBlock + threadIdx.x;
-    const bool v = i < f.n && in_frustum(f, i);
-    if (i < f.n) flags[i] = v ? 1 : 0;
-    local += __syncthreads_count(v);
-  }
-  if (threadIdx.x == 0) counts[blockIdx.x] = local;
-}
-
-// One block: exclusive prefix over counts[0..nb) -> offsets, total -> *n_visible.
-__global__ void __launch_bounds__(1024) frustum_scan_kernel(const int32_t* counts, int32_t* offsets, int32_t nb,
-                                                            int32_t* n_visible) {
-  __shared__ int32_t part[1024];
-  const int per = (nb + blockDim.x - 1) / blockDim.x;
-  const int b0 = threadIdx.x * per;
-  int32_t sum = 0;
-  for (int j = 0; j < per; ++j)
-    if (b0 + j < nb) sum += counts[b0 + j];
-  part[threadIdx.x] = sum;
-  __syncthreads();
-  // Hillis-Steele inclusive scan of the per-thread sums
-  for (int o = 1; o < int(blockDim.x); o <<= 1) {
-    const int32_t add = threadIdx.x >= unsigned(o) ? part[threadIdx.x - o] : 0;
-    __syncthreads();
-    part[threadIdx.x] += add;
-    __syncthreads();
-  }
-  int32_t run = part[threadIdx.x] - sum;  // exclusive
-  for (int j = 0; j < per; ++j) {
-    if (b0 + j < nb) {
-      offsets[b0 + j] = run;
-      run += counts[b0 + j];
-    }
-  }
-  if (threadIdx.x == blockDim.x - 1) *n_visible = part[threadIdx.x];
-}
-
-__global__ void __launch_bounds__(kCompactBlock) frustum_scatter_kernel(int64_t n, const uint8_t* flags,
-                                                                        const int32_t* offsets, int32_t* idx) {
+// Visibility bits (word w: primitives 32 w .. 32 w + 31) and the count of each block's `rounds`
+// rounds of kCompactChunk primitives. A thread takes four neighbouring centres at once, as three
+// 16-byte loads (VEC: the centres are 16-byte aligned); eight threads make a word.
+template <bool VEC>
+__global__ void __launch_bounds__(kCompactBlock) frustum_count_kernel(FrustumArgs f, uint32_t* bits, int32_t* counts,
+                                                                      int rounds) {
   __shared__ int32_t warp_tot[kCompactBlock / 32];
-  const int64_t base = int64_t(blockIdx.x) * kCompactChunk;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int32_t run = offsets[blockIdx.x];
-  for (int r = 0; r < kCompactChunk / kCompactBlock; ++r) {
-    const int64_t i = base + r * kCompactBlock + threadIdx.x;
-    const bool v = i < n && flags[i] != 0;
-    const unsigned bal = __ballot_sync(0xffffffffu, v);
-    if (lane == 0) warp_tot[warp] = __popc(bal);
-    __syncthreads();
-    int32_t before = 0, round = 0;
+  const int lane = threadIdx.x & 31;
+  int32_t sum = 0;
+  for (int r = 0; r < rounds; ++r) {
+    const int64_t base = (int64_t(blockIdx.x) * rounds + r) * kCompactChunk;
+    if (base >= f.n) break;  // block-uniform
+    constexpr int kGroups = kCompactChunk / (4 * kCompactBlock);
+    float c[kGroups][12];
 #pragma unroll
-    for (int w = 0; w < kCompactBlock / 32; ++w) {
-      const int32_t t = warp_tot[w];
-      before += w < warp ? t : 0;
-      round += t;
+    for (int g = 0; g < kGroups; ++g) {
+      const int64_t i = base + 4 * (g * kCompactBlock + int(threadIdx.x));
+      if (VEC && i + 4 <= f.n) {
+        const float4* p = reinterpret_cast<const float4*>(f.means + 3 * i);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const float4 v = __ldg(p + q);
+          c[g][4 * q] = v.x;
+          c[g][4 * q + 1] = v.y;
+          c[g][4 * q + 2] = v.z;
+          c[g][4 * q + 3] = v.w;
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < 12; ++q) c[g][q] = 3 * i + q < 3 * f.n ? __ldg(f.means + 3 * i + q) : 0.f;
+      }
     }
-    if (v) idx[run + before + __popc(bal & ((1u << lane) - 1u))] = int32_t(i);
-    run += round;
+#pragma unroll
+    for (int g = 0; g < kGroups; ++g) {
+      const int64_t i = base + 4 * (g * kCompactBlock + int(threadIdx.x));
+      uint32_t word = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (i + q < f.n && in_frustum(f, c[g][3 * q], c[g][3 * q + 1], c[g][3 * q + 2])) word |= 1u << q;
+      sum += __popc(word);
+      word <<= 4 * (lane & 7);
+      word |= __shfl_xor_sync(0xffffffffu, word, 1);
+      word |= __shfl_xor_sync(0xffffffffu, word, 2);
+      word |= __shfl_xor_sync(0xffffffffu, word, 4);
+      if ((lane & 7) == 0 && i < f.n) bits[i >> 5] = word;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (lane == 0) warp_tot[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int32_t t = 0;
+#pragma unroll
+    for (int w = 0; w < kCompactBlock / 32; ++w) t += warp_tot[w];
+    counts[blockIdx.x] = t;
+  }
+}
+
+// Ordered scatter: the block's first place is the sum of the counts before it, each warp then
+// places its words' set bits (a round is one word per warp and step). The last block writes the total.
+__global__ void __launch_bounds__(kCompactBlock) frustum_scatter_kernel(int64_t n, const uint32_t* bits,
+                                                                        const int32_t* counts, int32_t* idx,
+                                                                        int32_t* n_visible, int rounds) {
+  constexpr int kWarps = kCompactBlock / 32, kWords = kCompactChunk / 32;
+  static_assert(kWords <= kCompactBlock, "one thread per word of a round");
+  __shared__ int32_t warp_tot[kWarps];
+  __shared__ int32_t first[kWords];
+  __shared__ uint32_t word[kWords];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int32_t sum = 0;
+  for (int b = threadIdx.x; b < int(blockIdx.x); b += kCompactBlock) sum += counts[b];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (lane == 0) warp_tot[warp] = sum;
+  __syncthreads();
+  int32_t run = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) run += warp_tot[w];
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *n_visible = run + counts[blockIdx.x];
+  const int64_t words = (n + 31) / 32;
+  for (int r = 0; r < rounds; ++r) {
+    const int64_t w0 = (int64_t(blockIdx.x) * rounds + r) * kWords;
+    if (w0 >= words) break;  // block-uniform
     __syncthreads();
+    // exclusive scan of the words' bit counts
+    uint32_t m = 0;
+    if (threadIdx.x < kWords && w0 + threadIdx.x < words) m = bits[w0 + threadIdx.x];
+    int32_t inc = __popc(m);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) warp_tot[warp] = inc;
+    __syncthreads();
+    int32_t before = run;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      before += w < warp ? warp_tot[w] : 0;
+      run += warp_tot[w];
+    }
+    if (threadIdx.x < kWords) {
+      first[threadIdx.x] = before + inc - __popc(m);
+      word[threadIdx.x] = m;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int j = warp; j < kWords; j += kWarps) {
+      const uint32_t v = word[j];
+      if ((v >> lane) & 1u) idx[first[j] + __popc(v & ((1u << lane) - 1u))] = int32_t((w0 + j) * 32 + lane);
+    }
   }
 }
 
 static int64_t compact_blocks(int64_t n) { return (n + kCompactChunk - 1) / kCompactChunk; }
+
+// Bound: the centres' bytes (12 of them per primitive, read once) and the launches. A count with a
+// block barrier per 256 primitives, a byte per primitive, a one-block scan and a scatter with
+// another barrier per 256 took 40 us for 6e6 centres; bits, four centres per thread, and a scatter
+// that sums the counts before it (at most 2048: larger n gives each block more rounds) take 15 us
+// (the bytes alone 13 us at the measured copy rate).
+static void launch_compact(const FrustumArgs& f, unsigned char* scratch, int32_t* idx, int32_t* n_visible,
+                           cudaStream_t s) {
+  uint32_t* bits = reinterpret_cast<uint32_t*>(scratch);
+  int32_t* counts = reinterpret_cast<int32_t*>(scratch + (f.n + 15) / 16 * 16);
+  const int64_t chunks = compact_blocks(f.n);
+  const int rounds = int((chunks + kCompactMaxBlocks - 1) / kCompactMaxBlocks);
+  const unsigned blocks = unsigned((chunks + rounds - 1) / rounds);
+  if (aligned(f.means, 16)) frustum_count_kernel<true><<<blocks, kCompactBlock, 0, s>>>(f, bits, counts, rounds);
+  else frustum_count_kernel<false><<<blocks, kCompactBlock, 0, s>>>(f, bits, counts, rounds);
+  frustum_scatter_kernel<<<blocks, kCompactBlock, 0, s>>>(f.n, bits, counts, idx, n_visible, rounds);
+}
 
 }  // namespace nasg
 
@@ -530,10 +597,6 @@ extern "C" nasg_status nasg_frustum_compact(int64_t n, const float* means, const
   if (!aligned(means, 4) || !aligned(idx, 4) || !aligned(n_visible, 4) || !aligned(workspace, 16))
     return NASG_ERR_ALIGN;
   if (workspace_bytes < nasg_frustum_workspace_bytes(n)) return NASG_ERR_RANGE;
-  const int64_t nb = compact_blocks(n);
-  uint8_t* flags = static_cast<uint8_t*>(workspace);
-  int32_t* counts = reinterpret_cast<int32_t*>(flags + (n + 15) / 16 * 16);
-  int32_t* offsets = counts + nb;
   FrustumArgs f{};
   f.means = means;
   f.n = n;
@@ -541,9 +604,7 @@ extern "C" nasg_status nasg_frustum_compact(int64_t n, const float* means, const
   for (int j = 0; j < 3; ++j) f.c[j] = center[j];
   f.t = tan_half_fov;
   f.near_z = near_z;
-  frustum_count_kernel<<<unsigned(nb), kCompactBlock, 0, s>>>(f, flags, counts);
-  frustum_scan_kernel<<<1, 1024, 0, s>>>(counts, offsets, int32_t(nb), n_visible);
-  frustum_scatter_kernel<<<unsigned(nb), kCompactBlock, 0, s>>>(n, flags, offsets, idx);
+  launch_compact(f, static_cast<unsigned char*>(workspace), idx, n_visible, s);
   return check_launch();
 }
 
@@ -692,8 +753,8 @@ extern "C" nasg_status nasg_train_state_refresh_bf16(const nasg_desc* desc, cons
 // a renderer plugged into a host application that owns every device allocation
 // through its own pool and forbids others, or a per-frame loop with a fixed
 // memory budget where a cudaMalloc would synchronise the device and stall the
-// frame. For them, nasg_frustum_compact_noalloc keeps its scratch (one
-// visibility byte per primitive, per-chunk counts and offsets) in a fixed
+// frame. For them, nasg_frustum_compact_noalloc keeps its scratch
+// (visibility bits, per-block counts; room for a byte per primitive and two words per chunk) in a fixed
 // array of this library's device memory instead of a caller-provided
 // workspace. The array is sized for NASG_NOALLOC_MAX_PRIMS primitives and is
 // held by every GPU that loads the library until the process exits.
@@ -745,12 +806,8 @@ extern "C" nasg_status nasg_frustum_compact_noalloc(int64_t n, const float* mean
   if (!aligned(means, 4) || !aligned(idx, 4) || !aligned(n_visible, 4)) return NASG_ERR_ALIGN;
   unsigned char* ws = noalloc_scratch();
   if (!ws) return NASG_ERR_CUDA;
-  // Every byte the kernels read is written earlier in the same call (flags for
-  // i < n, counts and offsets for the n's chunks), so nothing needs clearing.
-  const int64_t nb = compact_blocks(n);
-  uint8_t* flags = ws;
-  int32_t* counts = reinterpret_cast<int32_t*>(ws + (n + 15) / 16 * 16);
-  int32_t* offsets = counts + nb;
+  // Every byte the kernels read is written earlier in the same call (bits for
+  // i < n, counts for the n's blocks), so nothing needs clearing.
   FrustumArgs f{};
   f.means = means;
   f.n = n;
@@ -758,8 +815,6 @@ extern "C" nasg_status nasg_frustum_compact_noalloc(int64_t n, const float* mean
   for (int j = 0; j < 3; ++j) f.c[j] = center[j];
   f.t = tan_half_fov;
   f.near_z = near_z;
-  frustum_count_kernel<<<unsigned(nb), kCompactBlock, 0, s>>>(f, flags, counts);
-  frustum_scan_kernel<<<1, 1024, 0, s>>>(counts, offsets, int32_t(nb), n_visible);
-  frustum_scatter_kernel<<<unsigned(nb), kCompactBlock, 0, s>>>(n, flags, offsets, idx);
+  launch_compact(f, ws, idx, n_visible, s);
   return check_launch();
 }

@@ -1,13 +1,14 @@
 """The fused step's ways of moving master, m and v (16-byte copies shared by two lanes, 8-byte copies
-per lane).
+per lane) and the compaction's forms (16-byte and element loads, several rounds per block).
 
 The copies change no arithmetic, so a state whose planes are 16-byte aligned and the same state
 8 bytes further (which takes the 8-byte copies) end the same but for the compiler's
 contraction choices in the two kernels: a few ulps (2^-24 each) of the moments and of
-the update, under 1e-6 relative L2 per plane."""
+the update, under 1e-6 relative L2 per plane. Index lists are integers and equal."""
 import numpy as np
 import pytest
 
+from oracle import frustum as ofr
 from paper_2606_09794_gb300 import inputs
 from tests._parity import rel_l2
 
@@ -54,3 +55,23 @@ def test_copies_of_either_width_agree(lib, n, L, frame, loss):
     for p in range(ma.shape[0]):
         assert rel_l2(ma[p], mb[p]) <= 1e-6 and rel_l2(va[p], vb[p]) <= 1e-6
         assert np.abs(ta[p] - tb[p]).max() <= 1e-6 * max(1.0, np.abs(tb[p]).max())
+
+
+# one primitive, word and chunk edges, and more than 2048 chunks (two rounds per block)
+@pytest.mark.parametrize("n", [1, 31, 33, 4096, 4099, 300_001, 2048 * 4096 + 4097])
+def test_compaction_forms_agree(lib, n):
+    import torch
+    rng = np.random.default_rng(n)
+    means = rng.uniform(-1.5, 1.5, (n, 3)).astype(np.float32)
+    cam = inputs.shell_scene(2000, 1, 9, fov_sample=2000).cameras[2]
+    lists = []
+    for offset in (0, 1):
+        idx, nv = lib.nasg_frustum_compact(_at(means, offset), cam.rot, cam.center, cam.tan_half_fov * 0.5)
+        lists.append(idx[:int(nv.item())].cpu().numpy())
+    np.testing.assert_array_equal(lists[0], lists[1])
+    assert np.all(np.diff(lists[0]) > 0)
+    ref = ofr.visible(means, cam.rot, cam.center, cam.tan_half_fov * 0.5)
+    margin = ofr.boundary_margin(means, cam.rot, cam.center, cam.tan_half_fov * 0.5)
+    got = np.zeros(n, bool)
+    got[lists[0]] = True
+    assert not ((got != ref) & (margin > 1e-5)).any()

@@ -4,6 +4,7 @@
 
 #include <map>
 #include <mutex>
+#include <tuple>
 #include <utility>
 
 #include "nasg_host.h"
@@ -48,6 +49,21 @@ nasg_status ensure_smem_limit(const void* kernel, size_t bytes) {
     have = bytes;
   }
   return NASG_OK;
+}
+
+int blocks_per_sm(const void* kernel, int threads, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, const void*, int, size_t>, int> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  std::lock_guard<std::mutex> lock(mu);
+  int& nb = known[{dev, kernel, threads, smem}];
+  if (nb == 0) {
+    int v = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kernel, threads, smem) != cudaSuccess || v < 1) return 1;
+    nb = v;
+  }
+  return nb;
 }
 
 int sm_count() {

@@ -38,6 +38,11 @@ int* device_error_word();
 // NASG_ERR_CUDA.
 nasg_status ensure_smem_limit(const void* kernel, size_t bytes);
 
+// Blocks of `threads` threads and `smem` dynamic bytes of `kernel` that fit an SM of the current
+// device at once (at least 1), asked of the runtime once per (device, kernel, threads, smem): the
+// occupancy calculator costs more than a launch's other host work.
+int blocks_per_sm(const void* kernel, int threads, size_t smem);
+
 // Grid for a grid-stride loop over `items` with `block` threads: one item per
 // thread, capped so that a 64-bit item count never overflows the grid.
 inline unsigned grid_for(int64_t items, int block) {

@@ -667,12 +667,7 @@ constexpr int kEvalBlock = 256;
 
 template <typename K>
 unsigned persistent_grid(K kernel, int64_t threads, int block) {
-  static int per_sm = 0;  // per kernel instantiation
-  if (per_sm == 0) {
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, block, 0) != cudaSuccess || nb < 1) nb = 1;
-    per_sm = nb;
-  }
+  const int per_sm = blocks_per_sm(reinterpret_cast<const void*>(kernel), block, 0);
   const unsigned cap = unsigned(sm_count() * per_sm);
   const unsigned need = grid_for(threads, block);
   return need < cap ? need : cap;
@@ -713,9 +708,7 @@ nasg_status launch_tma_geom(const EvalArgs& a, cudaStream_t s) {
   const size_t smem = size_t(NS) * g.stage_bytes + barrier_bytes(NS) + (tanh_table<FRAME, T>() ? kTanhBytes : 0u);
   auto k = eval_tma_kernel<FRAME, T, MODE, FLAGS, ANYN, LC, KI, NS>;
   if (const nasg_status e = ensure_smem_limit(reinterpret_cast<const void*>(k), smem); e != NASG_OK) return e;
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NT, smem) != cudaSuccess || per_sm < 1)
-    per_sm = 1;
+  const int per_sm = blocks_per_sm(reinterpret_cast<const void*>(k), NT, smem);
   const uint32_t n_tiles = uint32_t((a.n + g.tp - 1) / g.tp);
   const uint32_t cap = uint32_t(sm_count() * per_sm);
   k<<<n_tiles < cap ? n_tiles : cap, NT, smem, s>>>(a);

@@ -385,8 +385,7 @@ static nasg_status launch_step_k(const StepArgs& s, cudaStream_t st) {
   constexpr size_t smem = step_smem_bytes<P, MOVE>();
   auto k = step_kernel<FRAME, IDX, MOVE, LOSS>;
   if (const nasg_status e = ensure_smem_limit(reinterpret_cast<const void*>(k), smem); e != NASG_OK) return e;
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+  const int per_sm = blocks_per_sm(reinterpret_cast<const void*>(k), 256, smem);
   const int64_t threads = s.e.n_items << s.e.slice_log2;
   const unsigned need = grid_for(threads, 256);
   const unsigned cap = unsigned(sm_count() * per_sm);

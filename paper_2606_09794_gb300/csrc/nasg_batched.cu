@@ -7,14 +7,14 @@
 // scheduling, by a 4-byte counter reset), so a stream capture of it records a
 // CUDA graph that can be replayed. Work items are tiles of k sub-tiles of
 // I x 256/S primitives of one scene (S = lanes per primitive for that scene's L,
-// I = unit_items: a thread evaluates I items of each sub-tile one after the other).
+// I = batch_items: a thread evaluates I items of each sub-tile one after the other).
 // Blocks take tiles round-robin (static) or from an atomic counter (dynamic),
 // look the scene up in the shared-memory copy of the table, and evaluate the
 // tile with the lobe-pair lanes of the single-scene kernels, fetching each
 // lane's next sub-tile item before computing the current one. No thread waits
 // on another block. A staged variant moves each sub-tile's parameter spans,
 // means, upstream gradients and diffuse colours into shared memory with bulk
-// copies (span plans for any N), three sub-tiles ahead (one elected producer
+// copies (span plans for any N), two (BF16) or three (FP32) sub-tiles ahead (one elected producer
 // thread, full/empty mbarriers, every wait bounded), for the scenes whose planes
 // allow it (L >= 4), and loads the rest directly; its copy of the
 // scene table sits in dynamic shared memory, sized for the batch. The autotuner times the candidate schedules on the
@@ -34,7 +34,7 @@ struct SceneDev {
   int32_t staged;  // bit 0: parameter spans may be moved by bulk copies (even L >= 4, N L sizeof(T) % 16 == 0,
                    // 16-byte aligned planes); bit 1: the means, upstream gradients and diffuse colours
                    // too (16-byte aligned buffers, moved by span plans)
-  int32_t pad;
+  int32_t items;   // items per thread in a sub-tile (I), the same for the whole batch
 };
 
 constexpr int kMaxScenes = NASG_MAX_SCENES;
@@ -114,6 +114,23 @@ __device__ __forceinline__ void eval_scene_item(const EvalArgs& a, const RawItem
 // then as given (the table is internal; each record holds its scene's own buffers).
 inline int lobe_class(int32_t L) { return L == 4 ? 0 : (L == 8 ? 1 : (L == 16 ? 2 : 3)); }
 
+// Items per thread in a sub-tile. BF16: three, so that the wait for a stage, the producer's turn
+// and the scene's lookup are shared by three items, while that leaves each block of two per SM
+// at least eight sub-tiles; else two (a last round of large sub-tiles leaves more blocks idle). 16
+// scenes of 1.05e7 primitives: 1311 us unrolled with two items and three stages, 1252 us not
+// unrolled, 1242 us with two stages, 1217 us with three items; 6 scenes of up to 3e5: 111, 107, 105,
+// 104 us; 3 scenes of 75 000 primitives: 10.4 us with two items, 12.4 us with three.
+static int batch_items(const nasg_scene* scenes, int32_t n_scenes, int32_t param_dtype) {
+  if (param_dtype != NASG_DTYPE_BF16) return unit_items<float>();
+  const int most = unit_items<__nv_bfloat16>();
+  const int64_t enough = int64_t(sm_count()) * 2 * 8 * 256 * most;  // lanes
+  int64_t lanes = 0;
+  for (int j = 0; j < n_scenes && lanes < enough; ++j)
+    if (scenes[j].n > 0 && scenes[j].n_lobes >= 1 && scenes[j].n_lobes <= NASG_MAX_LOBES)
+      lanes += std::min<int64_t>(scenes[j].n, enough) << slice_log2(scenes[j].n_lobes);
+  return lanes >= enough ? most : most - 1;
+}
+
 // FLAGS: kFlagsDefault (raw activations, approximate normalisation) or
 // kFlagsRuntime (modes read from the arguments).
 template <int FRAME, typename T, int FLAGS, bool PAIRS>
@@ -145,7 +162,7 @@ __global__ void __launch_bounds__(256, 2) batched_kernel(const BatchArgs b) {
     const int tp = 256 >> sc.slice_log2;
     const int local = threadIdx.x >> sc.slice_log2;
     const int l0 = 2 * (threadIdx.x & ((1 << sc.slice_log2) - 1));
-    const int sub = b.sub_tiles * unit_items<T>();  // sub-items of tp primitives in the tile
+    const int sub = b.sub_tiles * sd[lo].items;  // sub-items of tp primitives in the tile
     const int64_t base = (tile - sd[lo].tile_begin) * int64_t(tp) * sub;
     RawItem<T, P> cur, nxt;
     fetch_scene_item<T, P>(sc, base + local, l0, true, cur);
@@ -178,9 +195,10 @@ struct PlanDev {
 // Staged variant
 // ---------------------------------------------------------------------------
 
-// Stages in flight per block.
+// Stages in flight per block: three for FP32; two for BF16, whose larger stages of three items then
+// still fit two blocks per SM.
 template <typename T>
-constexpr int batch_stages() { return 3; }
+constexpr int batch_stages() { return sizeof(T) == 2 ? 2 : 3; }
 constexpr int kMaxBatchStages = 3;
 constexpr uint32_t kUnitEnd = 0xffffffffu;
 
@@ -226,7 +244,7 @@ __device__ __forceinline__ bool issue_unit(const BatchArgs& b, const SceneDev* s
   const int32_t staged = sd[sc_i].staged;
   const int64_t n = sc.n;
   const uint32_t L = uint32_t(sc.n_lobes);
-  const int64_t tp = int64_t(256 >> sc.slice_log2) * unit_items<T>();
+  const int64_t tp = int64_t(256 >> sc.slice_log2) * sd[sc_i].items;
   const int64_t p0 = (u - sd[sc_i].unit_begin) * tp;
   const int64_t count = n - p0 < tp ? n - p0 : tp;
   meta->unit = unit;
@@ -345,9 +363,13 @@ __global__ void __launch_bounds__(kStagedThreads, 2) batched_staged_kernel(const
     pending &= ~(1u << s);  // this stage's fill (whoever issued it) has landed
     const StageMeta m = meta[s];
     if (m.unit == kUnitEnd) break;  // block-uniform: every warp reads the same stage
-    const EvalArgs& sc = sd[m.scene >= 0 ? m.scene : 0].args;
-#pragma unroll
-    for (int k = 0; k < unit_items<T>(); ++k) {
+    const SceneDev& scene = sd[m.scene >= 0 ? m.scene : 0];
+    const EvalArgs& sc = scene.args;
+    // not unrolled: copies of the item's code for each of the lobe-count classes do not fit the
+    // instruction cache (0.85 of 8 stall cycles per issue were for want of instructions)
+    const int items = unit_items<T>() == 1 ? 1 : scene.items;
+#pragma unroll 1
+    for (int k = 0; k < items; ++k) {
       RawItem<T, P> r;
       r.ok = 0;
       int64_t prim = 0;
@@ -395,7 +417,7 @@ __global__ void __launch_bounds__(kStagedThreads, 2) batched_staged_kernel(const
           fetch_scene_item<T, P>(sc, prim, l0, loc < m.count, r);
         }
       }
-      if (k == unit_items<T>() - 1) {
+      if (k == items - 1) {
         __syncwarp();
         if ((threadIdx.x & 31) == 0) mbar_arrive(&empty[s]);  // this warp is done with the stage
       }
@@ -441,6 +463,7 @@ extern "C" nasg_status nasgabor_batched_prepare(const nasg_scene* scenes, int32_
     return lobe_class(scenes[x].n_lobes) < lobe_class(scenes[y].n_lobes);
   });
   int64_t tiles = 0, prims = 0, lobes = 0;
+  const int items = batch_items(scenes, n_scenes, modes->param_dtype);
   bool pair_path = true;
   for (int j = 0; j < n_scenes; ++j) {
     const nasg_scene& s = scenes[order[j]];
@@ -490,8 +513,8 @@ extern "C" nasg_status nasgabor_batched_prepare(const nasg_scene* scenes, int32_
                    : 0;
     d.tile_begin = tiles;
     d.unit_begin = tiles * sub_tiles;
-    d.pad = 0;
-    const int64_t tile_prims = int64_t(256 >> a.slice_log2) * unit_items_of(modes->param_dtype) * sub_tiles;
+    d.items = items;
+    const int64_t tile_prims = int64_t(256 >> a.slice_log2) * items * sub_tiles;
     tiles += (s.n + tile_prims - 1) / tile_prims;
     prims += s.n;
     lobes += s.n * s.n_lobes;

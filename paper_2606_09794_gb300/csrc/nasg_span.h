@@ -168,11 +168,11 @@ NASG_HD SpanPlan tile_span(const TileGeom& g, uint32_t n, uint32_t n_lobes, uint
   return span_plan((uint64_t(c) * n + p0) * es, count * es, uint64_t(3) * n * es);
 }
 
-// Items per thread in a sub-tile of the batched kernels: two for BF16 parameters
-// (sub-tiles of 2 x 256/S primitives), one for FP32 (whose stages are twice as large).
+// The most items per thread in a sub-tile of the batched kernels: three for BF16 parameters
+// (sub-tiles of 3 x 256/S primitives; two for batches of few sub-tiles), one for FP32 (whose
+// stages are twice as large).
 template <typename T>
-NASG_HD constexpr int unit_items() { return sizeof(T) == 2 ? 2 : 1; }
-NASG_HD constexpr int unit_items_of(int param_dtype) { return param_dtype == 1 ? 2 : 1; }  // NASG_DTYPE_BF16
+NASG_HD constexpr int unit_items() { return sizeof(T) == 2 ? 3 : 1; }
 
 // Stage layout of the staged batched kernel: room for the sub-tile of any scene it
 // stages (L >= 4, so S >= 2: at most I x 128 primitives and I x 512 lobes), i.e. the

@@ -35,6 +35,8 @@ struct EvalArgs {
   int32_t n_lobes;
   int32_t slice;        // S = next_pow2(ceil(n_lobes / 2)) lanes per primitive
   int32_t slice_log2;
+  int32_t width;        // lanes per primitive in eval_kernel: S, or ceil(n_lobes / 2) where that
+                        // fits more primitives into a warp (see eval_width)
   int32_t identity;
   int32_t normalised;
   int32_t exact;        // exact normalisation (implies normalised)
@@ -196,22 +198,13 @@ struct RawItem {
   uint32_t i;   // primitive (IDX = uint32_t) -- see EvalItem for 64-bit
 };
 
-// Element offsets use IDX (uint32_t when P*N*L < 2^31, else uint64_t).
-// `total` is the number of lane items (items << slice_log2).
+// Element offsets use IDX (uint32_t when P*N*L < 2^31, else uint64_t). i: the primitive, or a
+// value of at least N for none.
 template <typename T, int P, typename IDX, bool EVEN, bool FWD, bool BWD>
-__device__ __forceinline__ void fetch_item(const EvalArgs& a, IDX total, IDX t, int l0, RawItem<T, P>& r,
-                                           IDX& prim) {
+__device__ __forceinline__ void fetch_prim(const EvalArgs& a, IDX i, int l0, RawItem<T, P>& r, IDX& prim) {
   const T* __restrict__ params = static_cast<const T*>(a.params);
   const IDX n = IDX(a.n);
   r.ok = 0;
-  if (t >= total) return;
-  const IDX item = t >> a.slice_log2;
-  IDX i = item;
-  if (a.idx) {
-    const int32_t v = __ldg(a.idx + item);
-    if (v < 0) return;  // out-of-range index entries are skipped
-    i = IDX(v);
-  }
   if (i >= n) return;
   r.ok = 1;
   prim = i;
@@ -246,6 +239,21 @@ __device__ __forceinline__ void fetch_item(const EvalArgs& a, IDX total, IDX t, 
       r.w[p] = *reinterpret_cast<typename RawWord<T>::type*>(&w);
     }
   }
+}
+
+// `total` is the number of lane items (items << slice_log2).
+template <typename T, int P, typename IDX, bool EVEN, bool FWD, bool BWD>
+__device__ __forceinline__ void fetch_item(const EvalArgs& a, IDX total, IDX t, int l0, RawItem<T, P>& r,
+                                           IDX& prim) {
+  r.ok = 0;
+  if (t >= total) return;
+  IDX i = t >> a.slice_log2;
+  if (a.idx) {
+    const int32_t v = __ldg(a.idx + i);
+    if (v < 0) return;  // out-of-range index entries are skipped
+    i = IDX(v);
+  }
+  fetch_prim<T, P, IDX, EVEN, FWD, BWD>(a, i, l0, r, prim);
 }
 
 __device__ __forceinline__ P2 unpack(float2 w) { P2 r; r.v = w; return r; }
@@ -285,9 +293,10 @@ constexpr int log2_of(int x) { return x <= 1 ? 0 : 1 + log2_of(x >> 1); }
 
 // LC: the lobe count when fixed at compile time (0: read from the arguments). C0_OWN: the
 // item holds only the diffuse colour of the lane's own output channel, in c0[0] (slices
-// of S >= 4 lanes, where a lane writes at most channel l0/2).
+// of S >= 4 lanes, where a lane writes at most channel l0/2). ANY_WIDTH: a.width neighbouring
+// lanes hold a primitive, any number of them.
 template <int FRAME, typename T, typename IDX, int MODE, bool EVEN, int FLAGS, int LC = 0, bool TAB = false,
-          bool C0_OWN = false>
+          bool C0_OWN = false, bool ANY_WIDTH = false>
 __device__ __forceinline__ void eval_item(const EvalArgs& a, const RawItem<T, FrameTraits<FRAME>::P>& cur, IDX i,
                                           int l0, const float4* tab = nullptr) {
   constexpr int P = FrameTraits<FRAME>::P;
@@ -353,6 +362,42 @@ __device__ __forceinline__ void eval_item(const EvalArgs& a, const RawItem<T, Fr
       }
     }
   }
+  if constexpr (ANY_WIDTH) {
+    // sums over `width` neighbouring lanes by halving, then from the first lane to all
+    const int lane = int(threadIdx.x & 31), g = l0 >> 1;
+    for (int w = a.width; w > 1;) {
+      const int h = (w + 1) >> 1;
+      const bool take = g + h < w;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if (FWD) {
+          const float y = __shfl_down_sync(0xffffffffu, rgb[c], h);
+          rgb[c] += take ? y : 0.f;
+        }
+        if (BWD) {
+          const float y = __shfl_down_sync(0xffffffffu, gd[c], h);
+          gd[c] += take ? y : 0.f;
+        }
+      }
+      w = h;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      if (FWD) rgb[c] = __shfl_sync(0xffffffffu, rgb[c], lane - g);
+      if (BWD) gd[c] = __shfl_sync(0xffffffffu, gd[c], lane - g);
+    }
+    if (ok) {
+      const float dot = BWD ? dot3_rn(gd, d) : 0.f;
+      for (int c = g; c < 3; c += a.width) {
+        if (FWD) a.rgb[3 * i + c] = pick3(rgb, c) + pick3(cur.c0, c);
+        if (BWD) {
+          store1(a.g_c0 + c * n + i, pick3(cur.gc, c), acc);
+          if (a.g_means) store1(a.g_means + 3 * i + c, mean_grad_rn(pick3(gd, c), dot, pick3(d, c), inv_dist), acc);
+        }
+      }
+    }
+    return;
+  }
   if (FWD && BWD && S() >= 4) {  // warp-uniform
     // Reduce-scatter over the slice: the colour and dLoss/dd partials (and the
     // partial d . dLoss/dd, linear in them) are summed so that lane c < 3 of each
@@ -404,13 +449,27 @@ __device__ __forceinline__ void eval_item(const EvalArgs& a, const RawItem<T, Fr
   }
 }
 
+// Lanes per primitive of eval_kernel: the slice S, or just the ceil(L/2) lanes that hold lobes where
+// more of those groups fit a warp (L = 5, 6: ten primitives per warp instead of eight, 9 and 10: six
+// instead of four, 11 and 12: five, 17 to 20: three instead of two).
+constexpr int eval_width(int n_lobes, int slice) {
+  const int pairs = (n_lobes + 1) / 2;
+  return 32 / pairs > 32 / slice ? pairs : slice;
+}
+
 // Each lane evaluates two lobes (2g, 2g+1) of its primitive in packed FP32x2
-// arithmetic; a slice of S = next_pow2(ceil(L/2)) lanes covers the primitive.
+// arithmetic; a slice of S = next_pow2(ceil(L/2)) lanes covers the primitive, or (GROUPS) `width`
+// neighbouring lanes of a warp do.
 // EVEN (L even, planes 2-element aligned): one 2-element load / store per plane.
 // The grid is persistent (as many blocks as fit) and each thread fetches its
 // next item's raw words before computing the current one (two buffers used in
 // turn), so that the loads of one item overlap the arithmetic of the previous.
-template <int FRAME, typename T, typename IDX, int MODE, bool EVEN>
+// Bound: latency and issue (issue 49-50 %, 16 warps per SM), so idle lanes cost what busy ones do. Fused
+// pass, slices / groups: L = 5 (3e5 primitives, BF16) 52.1 / 44.5 us, L = 9 (3e5, FP32) 100.8 / 79.0 us,
+// L = 11 (2e5, BF16) 70.8 / 61.0 us, L = 17 (1e5, FP32) 68.7 / 55.0 us. Groups where the slice is full (L = 1 to 4, 7, 8)
+// would only add their index arithmetic (L = 1: 52.1 / 54.4 us, L = 3 by list 16.6 / 17.3 us). A list's
+// entry read one item earlier spills in the FP32 backward and gains nothing.
+template <int FRAME, typename T, typename IDX, int MODE, bool EVEN, bool GROUPS>
 __global__ void __launch_bounds__(256, 2) eval_kernel(const EvalArgs a) {
   constexpr int FLAGS = kFlagsRuntime;
   constexpr int P = FrameTraits<FRAME>::P;
@@ -422,22 +481,55 @@ __global__ void __launch_bounds__(256, 2) eval_kernel(const EvalArgs a) {
     fill_tanh_table(tab);
     __syncthreads();
   }
-  const int l0 = 2 * (threadIdx.x & (a.slice - 1));
-  const IDX total = IDX(a.n_items) << a.slice_log2;
-  const IDX stride = IDX(gridDim.x) * blockDim.x;
   RawItem<T, P> b0, b1;
   IDX i0 = 0, i1 = 0;
-  IDX t0 = IDX(blockIdx.x) * blockDim.x;
-  fetch_item<T, P, IDX, EVEN, FWD, BWD>(a, total, t0 + threadIdx.x, l0, b0, i0);
-  // block-uniform loop: every lane of a warp reaches the shuffles
-  while (t0 < total) {
-    fetch_item<T, P, IDX, EVEN, FWD, BWD>(a, total, t0 + stride + threadIdx.x, l0, b1, i1);
-    eval_item<FRAME, T, IDX, MODE, EVEN, FLAGS, 0, TAB>(a, b0, i0, l0, tab);
-    t0 += stride;
-    if (t0 >= total) break;
-    fetch_item<T, P, IDX, EVEN, FWD, BWD>(a, total, t0 + stride + threadIdx.x, l0, b0, i0);
-    eval_item<FRAME, T, IDX, MODE, EVEN, FLAGS, 0, TAB>(a, b1, i1, l0, tab);
-    t0 += stride;
+  if constexpr (GROUPS) {
+    const int lane = threadIdx.x & 31, group = 32 / a.width;  // primitives per warp
+    const int sub = lane / a.width;
+    const int l0 = 2 * (lane - sub * a.width);
+    const IDX items = IDX(a.n_items);
+    const IDX stride = IDX(gridDim.x) * (256 / 32) * IDX(group);
+    // the warp's first item of a round; the lane's is `sub` later, none past the last group
+    IDX base = (IDX(blockIdx.x) * (256 / 32) + (threadIdx.x >> 5)) * IDX(group);
+    auto fetch = [&](IDX from, RawItem<T, P>& r, IDX& i) {
+      r.ok = 0;
+      const IDX item = from + IDX(sub);
+      if (sub >= group || item >= items) return;
+      IDX prim = item;
+      if (a.idx) {
+        const int32_t v = __ldg(a.idx + item);
+        if (v < 0) return;  // out-of-range index entries are skipped
+        prim = IDX(v);
+      }
+      fetch_prim<T, P, IDX, EVEN, FWD, BWD>(a, prim, l0, r, i);
+    };
+    fetch(base, b0, i0);
+    // warp-uniform loop: every lane of a warp reaches the shuffles
+    while (base < items) {
+      fetch(base + stride, b1, i1);
+      eval_item<FRAME, T, IDX, MODE, EVEN, FLAGS, 0, TAB, false, true>(a, b0, i0, l0, tab);
+      base += stride;
+      if (base >= items) break;
+      fetch(base + stride, b0, i0);
+      eval_item<FRAME, T, IDX, MODE, EVEN, FLAGS, 0, TAB, false, true>(a, b1, i1, l0, tab);
+      base += stride;
+    }
+  } else {
+    const int l0 = 2 * (threadIdx.x & (a.slice - 1));
+    const IDX total = IDX(a.n_items) << a.slice_log2;
+    const IDX stride = IDX(gridDim.x) * blockDim.x;
+    IDX t0 = IDX(blockIdx.x) * blockDim.x;
+    fetch_item<T, P, IDX, EVEN, FWD, BWD>(a, total, t0 + threadIdx.x, l0, b0, i0);
+    // block-uniform loop: every lane of a warp reaches the shuffles
+    while (t0 < total) {
+      fetch_item<T, P, IDX, EVEN, FWD, BWD>(a, total, t0 + stride + threadIdx.x, l0, b1, i1);
+      eval_item<FRAME, T, IDX, MODE, EVEN, FLAGS, 0, TAB>(a, b0, i0, l0, tab);
+      t0 += stride;
+      if (t0 >= total) break;
+      fetch_item<T, P, IDX, EVEN, FWD, BWD>(a, total, t0 + stride + threadIdx.x, l0, b0, i0);
+      eval_item<FRAME, T, IDX, MODE, EVEN, FLAGS, 0, TAB>(a, b1, i1, l0, tab);
+      t0 += stride;
+    }
   }
 }
 
@@ -673,18 +765,20 @@ unsigned persistent_grid(K kernel, int64_t threads, int block) {
   return need < cap ? need : cap;
 }
 
+template <int MODE, int FRAME, typename T, typename IDX, bool EVEN>
+nasg_status launch_idx_even(const EvalArgs& a, cudaStream_t s) {
+  constexpr int kBlock = kEvalBlock;
+  const bool groups = a.width != a.slice;
+  auto k = groups ? eval_kernel<FRAME, T, IDX, MODE, EVEN, true> : eval_kernel<FRAME, T, IDX, MODE, EVEN, false>;
+  const int64_t per_warp = 32 / a.width;
+  const int64_t threads = (a.n_items + per_warp - 1) / per_warp * 32;
+  k<<<persistent_grid(k, threads, kBlock), kBlock, 0, s>>>(a);
+  return check_launch();
+}
+
 template <int MODE, int FRAME, typename T, typename IDX>
 nasg_status launch_idx(const EvalArgs& a, bool even, cudaStream_t s) {
-  constexpr int kBlock = kEvalBlock;
-  const int64_t threads = a.n_items << a.slice_log2;
-  if (even) {
-    auto k = eval_kernel<FRAME, T, IDX, MODE, true>;
-    k<<<persistent_grid(k, threads, kBlock), kBlock, 0, s>>>(a);
-  } else {
-    auto k = eval_kernel<FRAME, T, IDX, MODE, false>;
-    k<<<persistent_grid(k, threads, kBlock), kBlock, 0, s>>>(a);
-  }
-  return check_launch();
+  return even ? launch_idx_even<MODE, FRAME, T, IDX, true>(a, s) : launch_idx_even<MODE, FRAME, T, IDX, false>(a, s);
 }
 
 // The TMA-staged kernel applies (see its requirements above).
@@ -754,7 +848,7 @@ nasg_status launch_frame_dtype(const EvalArgs& a, bool even, cudaStream_t s) {
   // 32-bit element offsets when every offset the kernel forms (P*N*L elements,
   // 3*N, and the thread index including one stride of prefetch) stays below 2^31.
   const int64_t NL = a.n * a.n_lobes;
-  const int64_t threads = a.n_items << a.slice_log2;
+  const int64_t threads = a.n_items << a.slice_log2;  // at least the register path's
   const int64_t lim = int64_t(1) << 31;
   const bool idx32 = NL * FrameTraits<FRAME>::P < lim && 3 * a.n < lim && 2 * threads + (int64_t(1) << 24) < lim;
   return idx32 ? launch_idx<MODE, FRAME, T, uint32_t>(a, even, s) : launch_idx<MODE, FRAME, T, uint64_t>(a, even, s);
@@ -788,6 +882,7 @@ nasg_status launch_eval(const nasg_desc* desc, EvalArgs a, cudaStream_t s) {
   a.dev_err = device_error_word();
   a.slice_log2 = slice_log2(desc->n_lobes);
   a.slice = 1 << a.slice_log2;
+  a.width = eval_width(desc->n_lobes, a.slice);
   const int es = elem_size(desc->param_dtype);
   const bool even = (desc->n_lobes % 2 == 0) && aligned(a.params, uintptr_t(2 * es)) &&
                     (a.g_params == nullptr || aligned(a.g_params, 8));

@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(THREADS, THREADS > 256 ? 2 : 4) depth_pass_ker
     key[i] = j < m ? kin[j] : sort::kNone;
     val[i] = FIRST ? j : (j < m ? vin[j] : 0u);
   }
-  const int cnt = sort::sort_block<THREADS, ITEMS>(s, ps, block, digit_base, key, val);
+  const int cnt = sort::sort_block<THREADS, ITEMS, LAST>(s, ps, block, digit_base, key, val);
   chain_next();
   const uint32_t mask = (1u << ps.bits) - 1u;
   for (int p = threadIdx.x; p < cnt; p += THREADS) {
@@ -655,7 +655,7 @@ __global__ void __launch_bounds__(THREADS, THREADS > 256 ? 2 : 4) list_pass_kern
     key[i] = p < size ? s.key[p] : sort::kNone;
     val[i] = p < size ? s.val[p] : 0u;
   }
-  const int cnt = sort::sort_block<THREADS, ITEMS>(s, ps, block, digit_base, key, val);
+  const int cnt = sort::sort_block<THREADS, ITEMS, true>(s, ps, block, digit_base, key, val);
   chain_next();
   write_pairs<THREADS, ITEMS, LAST>(s, ps, cnt, kout, vout, ranges, a.x_bits, a.tiles_x);
 }
@@ -680,7 +680,7 @@ __global__ void __launch_bounds__(THREADS, THREADS > 256 ? 2 : 4) pair_pass_kern
     key[i] = j < m ? kin[j] : sort::kNone;
     val[i] = j < m ? vin[j] : 0u;
   }
-  const int cnt = sort::sort_block<THREADS, ITEMS>(s, ps, block, digit_base, key, val);
+  const int cnt = sort::sort_block<THREADS, ITEMS, false>(s, ps, block, digit_base, key, val);
   chain_next();
   write_pairs<THREADS, ITEMS, LAST>(s, ps, cnt, kout, vout, ranges, x_bits, tiles_x);
 }

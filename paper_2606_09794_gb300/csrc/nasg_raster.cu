@@ -940,7 +940,11 @@ __global__ void __launch_bounds__(TileShape<PX>::NT) render_bwd_kernel(
 #pragma unroll
         for (int p = 0; p < PX; ++p) {
           if (al[p] > 0.f) {
-            const float inv = 1.f / (1.f - al[p]);
+            // 1/(1 - alpha), 1 - alpha in [0.01, 1]: the approximation and one Newton step, against 64
+            // bits no further off than the division (g_opacity 1.01e-6 either way at 1080p, without the
+            // pixels whose stop differs) and a third of its instructions: 489 -> 432 us
+            const float om = 1.f - al[p], r0 = rcpa(om);
+            const float inv = fmaf(r0, fmaf(-om, r0, 1.f), r0);
             const float Tb = T[p] * inv;  // transmittance in front of this contribution
             const float w = al[p] * Tb;
             gc0 = fmaf(w, g0[p], gc0);

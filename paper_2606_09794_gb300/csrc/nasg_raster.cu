@@ -459,7 +459,8 @@ __global__ void __launch_bounds__(THREADS, THREADS > 256 ? 2 : 4) depth_pass_ker
 
 // Exclusive scan, in depth order, of the tiles each drawn primitive reaches: its first pair. Notes
 // for every kStartGrain-th pair the primitive it belongs to, and the total; clears the pair passes'
-// states (as far as these pairs need them) on the way.
+// states (as far as these pairs need them) on the way. It runs before the host has compared the
+// squares' pairs with the capacity: where they exceed it, nothing sized by the capacity is written.
 __global__ void __launch_bounds__(kBlock) offsets_kernel(Header* hdr, uint32_t* ticket, int* err,
                                                          unsigned long long cap,
                                                          ulonglong2* __restrict__ pair_states,
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(kBlock) offsets_kernel(Header* hdr, uint32_t* 
 #pragma unroll
   for (int i = 0; i < kScanItems; ++i) {
     first[i] = run;
-    if (k0 + i < n) {
+    if (k0 + i < n && squares <= cap) {  // a forward that will be refused has no room in starts
       for (uint64_t b = (uint64_t(run) + kStartGrain - 1) / kStartGrain; b * kStartGrain < uint64_t(run) + c[i]; ++b)
         starts[b] = k0 + i;
     }

@@ -102,3 +102,60 @@ def test_binning_forms(lib, w, h, n, log_scale, depths):
     # lists that differ in order would differ in the image; a second run gives the same bits
     again, _ = r.forward(*[_dev(x) for x in sc])
     torch.testing.assert_close(again, img, rtol=0, atol=0)
+
+
+def _frame(lib, n, w, h, seed):
+    rng = np.random.default_rng(seed)
+    sc = [rng.uniform(-1, 1, (n, 3)), np.exp(rng.uniform(-4.0, -1.8, (n, 3))), rng.normal(size=(n, 4)),
+          rng.uniform(0.02, 0.98, n), rng.uniform(0, 1, (n, 3))]
+    sc = [x.astype(np.float32) for x in sc]
+    fx = np.float32(0.5 * max(w, h) / 0.4)
+    cam = lib.raster_camera(np.eye(3), (0.0, 0.0, -4.0), w, h, fx)
+    ocam = {"rot": np.eye(3), "centre": np.array([0.0, 0.0, -4.0]), "fx": fx, "fy": fx, "cx": 0.5 * w, "cy": 0.5 * h,
+            "near": np.float32(0.2)}
+    r = lib.Raster(n, cam, 1 << 23)
+    dev = [_dev(x) for x in sc]
+    img, T = r.forward(*dev)
+    return r, sc, dev, T, ocam, rng
+
+
+# an infinite or NaN upstream gradient at one pixel reaches the primitives that contribute there, an
+# infinite colour those in front of it at the pixels it contributes to, and no others
+@pytest.mark.parametrize("w,h,n", [(432, 416, 1500), (40, 16, 200)])
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_backward_keeps_non_finite_values_where_they_are(lib, w, h, n, bad):
+    r, sc, dev, T, ocam, rng = _frame(lib, n, w, h, 78)
+    g = rng.normal(size=(h, w, 3)).astype(np.float32)
+    px, py = w // 2 + 3, h // 2 - 2
+    ref_c, ref_o = (x.cpu().numpy() for x in r.backward(dev[4], T, _dev(g)))
+    g[py, px] = bad
+    gc, go = (x.cpu().numpy() for x in r.backward(dev[4], T, _dev(g)))
+    z, mean2, sigma2, valid = orr.project(*sc[:3], ocam)
+    alpha, _ = orr._alphas(px + 0.5, py + 0.5, mean2, sigma2, sc[3])
+    may = valid & (alpha >= (1 - MARGIN) * orr.ALPHA_MIN)   # all that could contribute at the pixel
+    touched = ~np.isfinite(gc).all(1)
+    assert touched.any() and not (touched & ~may).any()
+    assert not ((~np.isfinite(go)) & ~may).any()
+    assert rel_l2(gc[~may], ref_c[~may]) <= 1e-5 and rel_l2(go[~may], ref_o[~may]) <= 1e-5
+
+
+def test_refused_forward_stays_inside_its_workspace(lib):
+    """64 primitives over 65,536 tiles each, room for 16 pairs: the call is refused, the pair count
+    reported, and nothing past the workspace's end written, where the tables of 4.2e6 pairs would lie."""
+    import torch
+    n, w, h = 64, 4096, 4096
+    cam = lib.raster_camera(np.eye(3), (0.0, 0.0, -4.0), w, h, 5000.0)
+    r = lib.Raster(n, cam, 16)
+    nbytes = r.workspace.numel()
+    buf = torch.full((nbytes + (1 << 22),), 0xA5, dtype=torch.uint8, device="cuda")
+    r.workspace = buf[:nbytes]
+    means = torch.zeros((n, 3), device="cuda")
+    scales = torch.full((n, 3), 50.0, device="cuda")
+    quats = torch.tensor([[1.0, 0.0, 0.0, 0.0]], device="cuda").repeat(n, 1)
+    image = torch.full((h, w, 3), 7.0, device="cuda")
+    with pytest.raises(lib.NasgError) as e:
+        r.forward(means, scales, quats, torch.full((n,), 0.5, device="cuda"), torch.ones((n, 3), device="cuda"), image=image)
+    assert e.value.status == -7
+    torch.cuda.synchronize()
+    assert bool((buf[nbytes:] == 0xA5).all())
+    assert bool((image == 7.0).all())

@@ -92,7 +92,9 @@ struct ShArgs {
   float* g_means;
 };
 
-template <int DEG>
+// Bound: HBM (216 B per primitive at degree 3). STREAM: the coefficients are read as lines to be
+// evicted first, so that the read stream does not push the rest of L2 out.
+template <int DEG, bool STREAM>
 __global__ void __launch_bounds__(256) sh_fwd_kernel(const ShArgs a) {
   constexpr int NB = (DEG + 1) * (DEG + 1);
   const int64_t n = a.n;
@@ -106,7 +108,10 @@ __global__ void __launch_bounds__(256) sh_fwd_kernel(const ShArgs a) {
 #pragma unroll
     for (int j = 0; j < NB; ++j) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) rgb[c] = fmaf(__ldg(a.coeffs + (int64_t(j) * 3 + c) * n + i), Y[j], rgb[c]);
+      for (int c = 0; c < 3; ++c) {
+        const float* k = a.coeffs + (int64_t(j) * 3 + c) * n + i;
+        rgb[c] = fmaf(STREAM ? __ldcs(k) : __ldg(k), Y[j], rgb[c]);
+      }
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) a.rgb[3 * i + c] = rgb[c];
@@ -162,11 +167,17 @@ template <bool BWD>
 static nasg_status launch_sh(int degree, const ShArgs& a, cudaStream_t s) {
   constexpr int kBlock = 256;
   const unsigned grid = grid_for(a.n, kBlock);
+  // Coefficients that do not fit L2 (129 MB) beside the rest are streamed: degree 3 of 1e6 (192 MB)
+  // 39.0 -> 34.5 us, degree 2 of 1e6 (108 MB) 24.3 -> 20.7 us; smaller ones may be in L2 and should
+  // stay there for the next pass (degree 3 of 1e5, 19 MB, again and again: 5.3 us, streamed 8.2 us). The
+  // backward, which writes as much as it reads, is slower streamed (67 -> 72 us).
+  const bool stream = a.n * int64_t(12) * (degree + 1) * (degree + 1) >= int64_t(100) * 1000 * 1000;
   switch (degree) {
 #define NASG_SH_CASE(D)                                                   \
   case D:                                                                 \
     if (BWD) sh_bwd_kernel<D><<<grid, kBlock, 0, s>>>(a);                 \
-    else sh_fwd_kernel<D><<<grid, kBlock, 0, s>>>(a);                     \
+    else if (stream) sh_fwd_kernel<D, true><<<grid, kBlock, 0, s>>>(a);   \
+    else sh_fwd_kernel<D, false><<<grid, kBlock, 0, s>>>(a);              \
     break;
     NASG_SH_CASE(0)
     NASG_SH_CASE(1)

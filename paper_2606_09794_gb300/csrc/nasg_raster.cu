@@ -1088,10 +1088,10 @@ inline bool wait_total(const HostTotal* words, unsigned long long call, cudaStre
   return true;
 }
 
-// Launches a kernel of the chain: it may start while its predecessor runs (see chain_wait).
+// Launches a kernel of the chain: with `chain` it may start while its predecessor runs (see chain_wait).
 template <typename... P, typename... A>
-nasg_status launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
-                           const A&... args) {
+nasg_status launch_chained(bool chain, void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem,
+                           cudaStream_t s, const A&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(threads);
@@ -1101,7 +1101,7 @@ nasg_status launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = chain ? 1 : 0;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
   if (e != cudaSuccess) {
     record_cuda_error(e);
@@ -1115,7 +1115,7 @@ template <int THREADS, int ITEMS, typename K, typename... A>
 nasg_status launch_sort(K kernel, unsigned grid, cudaStream_t s, const A&... args) {
   constexpr size_t smem = sizeof(sort::Block<THREADS, ITEMS>);
   if (const nasg_status e = ensure_smem_limit(reinterpret_cast<const void*>(kernel), smem); e != NASG_OK) return e;
-  return launch_chained(kernel, grid, THREADS, smem, s, args...);
+  return launch_chained(true, kernel, grid, THREADS, smem, s, args...);
 }
 
 template <int THREADS, int ITEMS>
@@ -1233,7 +1233,7 @@ extern "C" nasg_status nasg_raster_forward(int64_t n, const float* means, const 
                               : depth_sort<kSmallThreads, kSmallItems>(ps, hdr, dkeys, order, uint32_t(n), s);
     if (e != NASG_OK) return e;
     constexpr int64_t kChunk = kBlock * kScanItems;
-    e = launch_chained(offsets_kernel, unsigned((n + kChunk - 1) / kChunk), kBlock, 0, s, hdr,
+    e = launch_chained(true, offsets_kernel, unsigned((n + kChunk - 1) / kChunk), kBlock, 0, s, hdr,
                        hdr->tickets + kDepthPasses, ps.err, (unsigned long long)(max_pairs),
                        reinterpret_cast<ulonglong2*>(ws + L.pair_states),
                        reinterpret_cast<unsigned long long*>(ws + L.scan_states), order[kDepthPasses & 1], reach,
@@ -1259,10 +1259,10 @@ extern "C" nasg_status nasg_raster_forward(int64_t n, const float* means, const 
   const uint32_t* list = vals[td.passes & 1];
   auto* ncontrib = at(L.ncontrib);
   if (two_pixels(tiles))
-    return launch_chained(render_fwd_kernel<2>, unsigned(tiles), TileShape<2>::NT, 0, s, cam, hdr, ranges, list, splat,
-                          colours, image, final_t, ncontrib);
-  return launch_chained(render_fwd_kernel<1>, unsigned(tiles), TileShape<1>::NT, 0, s, cam, hdr, ranges, list, splat,
-                        colours, image, final_t, ncontrib);
+    return launch_chained(n > 0, render_fwd_kernel<2>, unsigned(tiles), TileShape<2>::NT, 0, s, cam, hdr, ranges, list,
+                          splat, colours, image, final_t, ncontrib);
+  return launch_chained(n > 0, render_fwd_kernel<1>, unsigned(tiles), TileShape<1>::NT, 0, s, cam, hdr, ranges, list,
+                        splat, colours, image, final_t, ncontrib);
 }
 
 extern "C" nasg_status nasg_raster_backward(int64_t n, const float* colours, const nasg_raster_camera* camera,

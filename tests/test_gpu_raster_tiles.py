@@ -159,3 +159,18 @@ def test_refused_forward_stays_inside_its_workspace(lib):
     torch.cuda.synchronize()
     assert bool((buf[nbytes:] == 0xA5).all())
     assert bool((image == 7.0).all())
+
+
+def test_forward_under_capture(lib):
+    """Without primitives a forward needs no wait and can be captured."""
+    import torch
+    cam = lib.raster_camera(np.eye(3), (0.0, 0.0, -4.0), 40, 24, 50.0)
+    empty = lib.Raster(0, cam, 16)
+    e3, image, T = torch.empty((0, 3), device="cuda"), torch.ones((24, 40, 3), device="cuda"), torch.zeros((24, 40), device="cuda")
+    args = (e3, e3, torch.empty((0, 4), device="cuda"), torch.empty(0, device="cuda"), e3)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        empty.forward(*args, image=image, final_t=T)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert float(image.abs().max()) == 0.0 and float(T.min()) == 1.0

@@ -571,7 +571,7 @@ struct ListArgs {
   int tiles_x;
 };
 
-// First pass of the pair sort, 146 us of emission and 211 us of its radix pass before, 132 us now
+// First pass of the pair sort, 146 us of emission and 211 us of its radix pass before, 106 us now
 // (1e6 primitives at 1080p). A block's pairs are places [base, base + THREADS ITEMS) of the depth
 // order's list: it finds the primitives that hold them in `starts` and writes their tiles into
 // shared memory itself, so the list never goes through memory unsorted. A thread lists a
@@ -1016,9 +1016,10 @@ __global__ void __launch_bounds__(TileShape<PX>::NT) render_bwd_kernel(
 
 // One pixel per lane gives each tile twice the warps, which hides the chain through a pixel's
 // list where the image has few tiles. Backward alone, one / two pixels per lane: 60 tiles (1e5
-// primitives) 134 / 186 us, 240 tiles 106 / 136, 510 tiles 116 / 128, 920 tiles 135 / 119,
-// 2040 tiles 211 / 187, 8160 tiles 652 / 508: the line at four tiles per SM.
-inline bool two_pixels(int64_t tiles) { return tiles >= int64_t(4) * sm_count(); }
+// primitives) 114 / 152 us, 240 tiles 89 / 114, 510 tiles 99 / 109, 920 tiles 116 / 99, 8160 tiles
+// 540 / 414: the line at four tiles per SM. Whole forward: 510 tiles 202 / 209, 920 tiles 183 / 195,
+// 2040 tiles 237.2 / 236.8 and 167 / 162, 3600 tiles 283 / 270, 8160 tiles 595 / 559: at eight.
+inline bool two_pixels(int64_t tiles, int per_sm) { return tiles >= int64_t(per_sm) * sm_count(); }
 
 inline Cam make_cam(const nasg_raster_camera* c) {
   Cam k;
@@ -1258,7 +1259,7 @@ extern "C" nasg_status nasg_raster_forward(int64_t n, const float* means, const 
   }
   const uint32_t* list = vals[td.passes & 1];
   auto* ncontrib = at(L.ncontrib);
-  if (two_pixels(tiles))
+  if (two_pixels(tiles, 8))
     return launch_chained(n > 0, render_fwd_kernel<2>, unsigned(tiles), TileShape<2>::NT, 0, s, cam, hdr, ranges, list,
                           splat, colours, image, final_t, ncontrib);
   return launch_chained(n > 0, render_fwd_kernel<1>, unsigned(tiles), TileShape<1>::NT, 0, s, cam, hdr, ranges, list,
@@ -1291,7 +1292,7 @@ extern "C" nasg_status nasg_raster_backward(int64_t n, const float* colours, con
   const auto* ranges = reinterpret_cast<const uint2*>(ws + L.ranges);
   const auto* splat = reinterpret_cast<const Splat*>(ws + L.splat);
   const auto* ncontrib = reinterpret_cast<const uint32_t*>(ws + L.ncontrib);
-  if (two_pixels(tiles))
+  if (two_pixels(tiles, 4))
     render_bwd_kernel<2><<<unsigned(tiles), TileShape<2>::NT, 0, s>>>(cam, hdr, ranges, vals, splat, colours, final_t,
                                                                       ncontrib, g_image, g_colours, g_opacity);
   else

@@ -1046,16 +1046,29 @@ inline bool camera_ok(const nasg_raster_camera* c) {
          std::isfinite(c->centre[1]) && std::isfinite(c->centre[2]);
 }
 
+// While it lives, the thread's calls neither fail for nor end a capture that goes on elsewhere (page-locking,
+// its release and stream queries are refused during a capture in CUDA's default, global mode).
+struct BesideCaptures {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  BesideCaptures(const BesideCaptures&) = delete;
+  BesideCaptures& operator=(const BesideCaptures&) = delete;
+};
+
 // The page-locked words of one host thread and the number of its latest call, kept for the thread's
 // life (page-locking memory on every call would cost more than the call).
 struct HostWords {
   HostTotal* words = nullptr;
   unsigned long long calls = 0;
   ~HostWords() {
-    if (words) cudaFreeHost(words);
+    if (!words) return;
+    const BesideCaptures beside;
+    cudaFreeHost(words);
   }
   bool ready() {
     if (!words) {
+      const BesideCaptures beside;
       if (cudaHostAlloc(reinterpret_cast<void**>(&words), sizeof(HostTotal),
                         cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
         words = nullptr;
@@ -1071,6 +1084,7 @@ struct HostWords {
 // when the stream fails, is being captured, or finishes without it).
 inline bool wait_total(const HostTotal* words, unsigned long long call, cudaStream_t s, unsigned long long* pairs) {
   const volatile HostTotal* w = words;
+  const BesideCaptures beside;
   for (uint32_t spin = 1;; ++spin) {
     if (w->call == call) break;
     if (spin % 1024 != 0) continue;

@@ -20,9 +20,11 @@ def _dev(x):
 
 
 # (width, height, window corner and size, primitives, log-scale range): 27 x 26 = 702 and 700 x 1
-# tiles run two pixels per lane, the others one; the last list holds several staged batches
+# tiles run two pixels per lane in the backward, 37 x 33 = 1221 in the forward too, the others one;
+# the last list holds several staged batches
 @pytest.mark.parametrize("w,h,win,n,log_scale", [
     (432, 416, (201, 190, 33, 22), 300, (-4.5, -1.5)),
+    (592, 521, (281, 243, 33, 22), 300, (-4.5, -1.5)),
     (11193, 9, (5590, 0, 40, 9), 250, (-3.0, -1.5)),
     (37, 21, (0, 0, 37, 21), 300, (-4.5, -1.5)),
     (17, 1, (0, 0, 17, 1), 60, (-3.0, -1.0)),
@@ -174,3 +176,39 @@ def test_forward_under_capture(lib):
     graph.replay()
     torch.cuda.synchronize()
     assert float(image.abs().max()) == 0.0 and float(T.min()) == 1.0
+
+
+def test_forward_beside_a_capture(lib):
+    """A forward on another thread and stream, its first there, while this thread captures: neither
+    it nor that thread's end disturbs the capture."""
+    import threading
+
+    import torch
+    rng = np.random.default_rng(11)
+    n = 50
+    args = [_dev(x) for x in (rng.uniform(-1, 1, (n, 3)), np.full((n, 3), 0.05), rng.normal(size=(n, 4)),
+                              np.full(n, 0.5), rng.uniform(size=(n, 3)))]
+    cam = lib.raster_camera(np.eye(3), (0.0, 0.0, -4.0), 40, 24, 50.0)
+    want = lib.Raster(n, cam, 1 << 12).forward(*args)[0].clone()
+    beside, other = lib.Raster(n, cam, 1 << 12), torch.cuda.Stream()
+    image, T, x = torch.empty_like(want), torch.empty((24, 40), device="cuda"), torch.zeros(8, device="cuda")
+    errors = []
+
+    def run():
+        try:
+            beside.forward(*args, image=image, final_t=T, stream=other)
+        except Exception as e:  # reported below, after the capture has ended
+            errors.append(e)
+
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        x.add_(1.0)
+        thread = threading.Thread(target=run)
+        thread.start()
+        thread.join()
+        x.add_(1.0)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert not errors
+    assert torch.equal(image, want) and float(x.sum()) == 16.0

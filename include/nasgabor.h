@@ -505,7 +505,8 @@ size_t nasg_raster_workspace_bytes(int64_t n, int32_t width, int32_t height, int
  *   n_pairs: nullable host output, the number of (tile, primitive) pairs of the
  *          primitives' footprint squares (the lists hold those whose ellipse reaches
  *          the tile, a part of them).
- * The host waits once, for the projection (to size the sort). NASG_ERR_CAPACITY when
+ * The host waits once, for the projection (to size the sort), as the device's scheduling
+ * flags ask (polling, yielding or blocked). NASG_ERR_CAPACITY when
  * the pairs exceed max_pairs (n_pairs still reports the count); n < 2^31. A call that
  * returns an error after its first launch has waited for the stream: nothing of it is
  * running, and the workspace may be freed or used again on any stream. The lists'

@@ -36,6 +36,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstdint>
+#include <thread>
 
 #include "nasg_cover.h"
 #include "nasg_host.h"
@@ -1091,14 +1092,19 @@ inline nasg_status give_up(nasg_status why, cudaStream_t s) {
 }
 
 // Waits until the projection of call `call` has left its total (false with the CUDA error recorded
-// when the stream fails, is being captured, or finishes without it).
+// when the stream fails, is being captured, or finishes without it). The thread polls the word, as the
+// runtime's own waits do by default, or waits as the device's scheduling flags ask: yielding between polls,
+// or blocked until the stream is done. The flags are read once the first polls have failed.
 inline bool wait_total(const HostTotal* words, unsigned long long call, cudaStream_t s, unsigned long long* pairs) {
   const volatile HostTotal* w = words;
   const BesideCaptures beside;
+  unsigned schedule = 0;
   for (uint32_t spin = 1;; ++spin) {
     if (w->call == call) break;
+    if (schedule == cudaDeviceScheduleYield) std::this_thread::yield();
     if (spin % 1024 != 0) continue;
-    const cudaError_t e = cudaStreamQuery(s);
+    if (spin == 1024 && cudaGetDeviceFlags(&schedule) == cudaSuccess) schedule &= cudaDeviceScheduleMask;
+    const cudaError_t e = schedule == cudaDeviceScheduleBlockingSync ? cudaStreamSynchronize(s) : cudaStreamQuery(s);
     if (e == cudaErrorNotReady) {
       cudaGetLastError();  // no error
       continue;

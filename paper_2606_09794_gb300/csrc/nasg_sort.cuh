@@ -3,14 +3,15 @@
 // (decoupled look-back, Merrill & Garland 2016; as a radix pass, Adinets & Merrill 2022), so that
 // a pass reads and writes its data once, in one launch. A block takes its place from a ticket
 // counter: the blocks it looks back at have smaller tickets, so they are running or done, and
-// publish their own counts before they wait. Every wait is bounded (one second or kWaitLimit
-// polls); a block that gives up sets the library's device error word and `failed` in the
+// publish their own counts before they wait. Every wait is bounded (one second of waiting or
+// kWaitLimit polls); a block that gives up sets the library's device error word and `failed` in the
 // workspace's header, which later blocks and kernels read before they trust any list.
 #pragma once
 
 #include <stdint.h>
 
 #include "nasg_tma.cuh"
+#include "nasg_wait.h"
 
 namespace nasg {
 namespace sort {
@@ -39,11 +40,11 @@ __device__ __forceinline__ bool ready(unsigned long long v, uint32_t tag) {
 
 // Polls a predecessor's state until it is published; a state of kGone when it gave up.
 static __device__ __noinline__ unsigned long long wait_state(const unsigned long long* p, uint32_t tag, int* err) {
-  const uint64_t t0 = global_ns();
+  WaitClock clock(global_ns());
   for (uint32_t it = 1; it < kWaitLimit; ++it) {
     const unsigned long long v = ld_state(p);
     if (ready(v, tag)) return v;
-    if ((it & 255u) == 0 && global_ns() - t0 > kWaitNs) break;
+    if ((it & 255u) == 0 && clock.over(global_ns(), kWaitNs)) break;
   }
   if (err) atomicExch(err, NASG_DEVERR_WAIT_TIMEOUT);
   return kGone;

@@ -510,8 +510,9 @@ size_t nasg_raster_workspace_bytes(int64_t n, int32_t width, int32_t height, int
  * the pairs exceed max_pairs (n_pairs still reports the count); n < 2^31. A call that
  * returns an error after its first launch has waited for the stream: nothing of it is
  * running, and the workspace may be freed or used again on any stream. The lists'
- * device-side waits are bounded: should one give up, nasg_device_status() says so and
- * the image is empty.
+ * device-side waits are bounded: should one give up (the call has returned NASG_OK by
+ * then), nasg_device_status() says so, the image is empty, final_t is one and the
+ * gradients of nasg_raster_backward are zero.
  */
 nasg_status nasg_raster_forward(int64_t n, const float* means, const float* scales, const float* quats,
                                 const float* opacity, const float* colours, const nasg_raster_camera* camera,
@@ -568,6 +569,27 @@ double nasg_cosine_lr_factor(int64_t t, int64_t t_start, int64_t t_max);
  * library's failure detection without faulting or hanging the GPU.
  */
 nasg_status nasg_probe_wait_timeout(int32_t limit, void* stream);
+
+/*
+ * Diagnostics of the compositing sorts' waits. nasg_probe_look_back_timeout runs
+ * NASG_PROBE_LOOK_BACK_BLOCKS sort and scan blocks whose first predecessor publishes
+ * its counts (first = 0) or never does (first = 1): then each gives up after at most
+ * `limit` polls (1..2^20) per wait, and nasg_device_status() returns NASG_ERR_DEVICE.
+ *   results: device int32 [2 NASG_PROBE_LOOK_BACK_BLOCKS + 1]: entries each sort block
+ *            placed, counts before each scan block (-1 where it gave up), and the word
+ *            by which the forward's later kernels learn of it;
+ *   workspace: device, 8-byte aligned, >= NASG_PROBE_LOOK_BACK_BYTES.
+ * nasg_probe_raster_failed is nasg_raster_forward with that word set before its sorts
+ * (where = 1) or before its rendering (where = 2).
+ */
+#define NASG_PROBE_LOOK_BACK_BLOCKS 20
+#define NASG_PROBE_LOOK_BACK_BYTES 65536
+nasg_status nasg_probe_look_back_timeout(int32_t limit, int32_t first, int32_t* results, void* workspace,
+                                         size_t workspace_bytes, void* stream);
+nasg_status nasg_probe_raster_failed(int32_t where, int64_t n, const float* means, const float* scales,
+                                     const float* quats, const float* opacity, const float* colours,
+                                     const nasg_raster_camera* camera, float* image, float* final_t,
+                                     int64_t max_pairs, void* workspace, size_t workspace_bytes, void* stream);
 
 #ifdef __cplusplus
 }  /* extern "C" */

@@ -129,6 +129,9 @@ _decl("nasgabor_fused_fwd_bwd_host", [_P(NasgDesc), _vp, _vp, _vp, _P(ctypes.c_f
 _decl("nasg_raster_workspace_bytes", [_i64, _i32, _i32, _i64], ctypes.c_size_t)
 _decl("nasg_raster_forward", [_i64, _vp, _vp, _vp, _vp, _vp, _P(NasgRasterCamera), _vp, _vp, _i64, _vp,
                               ctypes.c_size_t, _P(_i64), _vp])
+_decl("nasg_probe_raster_failed", [_i32, _i64, _vp, _vp, _vp, _vp, _vp, _P(NasgRasterCamera), _vp, _vp, _i64, _vp,
+                                   ctypes.c_size_t, _vp])
+_decl("nasg_probe_look_back_timeout", [_i32, _i32, _vp, _vp, ctypes.c_size_t, _vp])
 _decl("nasg_raster_backward", [_i64, _vp, _P(NasgRasterCamera), _vp, _vp, _vp, _vp, _i64, _vp, ctypes.c_size_t,
                                _vp])
 
@@ -250,6 +253,22 @@ def nasg_cosine_lr_factor(t, t_max, t_start=0):
 def nasg_probe_wait_timeout(limit=1024, stream=None):
     """Diagnostic: run a bounded wait that cannot complete (sets the device error word)."""
     _check(lib.nasg_probe_wait_timeout(int(limit), _stream(stream)), "nasg_probe_wait_timeout")
+
+
+LOOK_BACK_BLOCKS = 20
+
+
+def nasg_probe_look_back_timeout(limit=1024, first=1, stream=None):
+    """Diagnostic: sort and scan blocks of the compositing lists whose first predecessor never publishes its
+    counts (first=1; 0: it does). Returns what each placed, the counts before each, and the failure word."""
+    results = torch.empty(2 * LOOK_BACK_BLOCKS + 1, device="cuda", dtype=torch.int32)
+    workspace = torch.empty(65536, device="cuda", dtype=torch.uint8)
+    s = torch.cuda.current_stream() if stream is None else stream
+    _check(lib.nasg_probe_look_back_timeout(int(limit), int(first), _ptr(results), _ptr(workspace), workspace.numel(),
+                                            _stream(s)), "nasg_probe_look_back_timeout")
+    s.synchronize()
+    r = results.tolist()
+    return r[:LOOK_BACK_BLOCKS], r[LOOK_BACK_BLOCKS:-1], r[-1]
 
 
 def lobe_planes(frame_mode="quat") -> int:
@@ -653,7 +672,9 @@ def raster_camera(rot, centre, width, height, fx, fy=None, cx=None, cy=None, nea
 class Raster:
     """Front-to-back compositing of primitives (see include/nasgabor.h) with a
     workspace sized for `max_pairs` (tile, primitive) pairs; forward keeps the
-    state that backward reuses."""
+    state that backward reuses. The lists' device-side waits are bounded: should one give
+    up, the image comes out empty and the gradients zero, and nasg_device_status() raises;
+    a program that must not go on with such a frame asks it."""
 
     def __init__(self, n, camera, max_pairs, device=None):
         self.n = int(n)
@@ -666,6 +687,7 @@ class Raster:
         self.n_pairs = None
 
     def forward(self, means, scales, quats, opacity, colours, image=None, final_t=None, stream=None):
+        """(image [h, w, 3], final_t [h, w])."""
         h, w = self.camera.height, self.camera.width
         dev = means.device
         for t, nm in ((means, "means"), (scales, "scales"), (quats, "quats"), (opacity, "opacity"),

@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(kBlock) offsets_kernel(Header* hdr, uint32_t* 
   if (t < 32) {
     if (t == 0) sort::st_state(states + block, (block == 0 ? sort::kAll : sort::kOwn) | sort::tag_bits(kTag) | total);
     unsigned long long before = 0;
-    const bool ok = block == 0 || sort::look_back_warp(states, block, kTag, err, &before);
+    const bool ok = block == 0 || sort::look_back_warp(states, block, kTag, kWaitLimit, err, &before);
     if (t == 0) {
       if (block > 0)
         sort::st_state(states + block,
@@ -1212,11 +1212,13 @@ extern "C" size_t nasg_raster_workspace_bytes(int64_t n, int32_t width, int32_t 
   return layout(n, tiles, int64_t(width) * height, max_pairs).total;
 }
 
-extern "C" nasg_status nasg_raster_forward(int64_t n, const float* means, const float* scales, const float* quats,
-                                           const float* opacity, const float* colours,
-                                           const nasg_raster_camera* camera, float* image, float* final_t,
-                                           int64_t max_pairs, void* workspace, size_t workspace_bytes,
-                                           int64_t* n_pairs, void* stream) {
+// `fail`: where the header's `failed` is set as by a wait that gave up (the probe's, else kNowhere).
+enum FailAt { kNowhere, kBeforeSorts, kBeforeRender };
+
+static nasg_status forward(FailAt fail, int64_t n, const float* means, const float* scales, const float* quats,
+                           const float* opacity, const float* colours, const nasg_raster_camera* camera, float* image,
+                           float* final_t, int64_t max_pairs, void* workspace, size_t workspace_bytes,
+                           int64_t* n_pairs, void* stream) {
   if (!camera) return NASG_ERR_NULL;
   if (!camera_ok(camera)) return NASG_ERR_RANGE;
   if (n < 0 || n >= (int64_t(1) << 31) || max_pairs < 0 || max_pairs >= (int64_t(1) << 32)) return NASG_ERR_RANGE;
@@ -1245,6 +1247,10 @@ extern "C" nasg_status nasg_raster_forward(int64_t n, const float* means, const 
   const TileDigits td = tile_digits(cam.tx, cam.ty);
 
   if (cudaMemsetAsync(ws + L.header, 0, L.head_end - L.header, s) != cudaSuccess) return check_launch();
+  auto set_failed = [&](FailAt where) {
+    return fail != where || cudaMemsetAsync(&hdr->failed, 1, 1, s) == cudaSuccess;
+  };
+  if (!set_failed(kBeforeSorts)) return give_up(check_launch(), s);
   unsigned long long total64 = 0;
   if (n > 0) {
     static thread_local HostWords host;
@@ -1259,6 +1265,7 @@ extern "C" nasg_status nasg_raster_forward(int64_t n, const float* means, const 
     ps.states = reinterpret_cast<unsigned long long*>(ws + L.depth_states);
     ps.failed = &hdr->failed;
     ps.err = device_error_word();
+    ps.limit = kWaitLimit;
     nasg_status e = n > kLargeDepth
                               ? depth_sort<kLargeThreads, kLargeItems>(ps, hdr, dkeys, order, uint32_t(n), s)
                               : depth_sort<kSmallThreads, kSmallItems>(ps, hdr, dkeys, order, uint32_t(n), s);
@@ -1281,12 +1288,14 @@ extern "C" nasg_status nasg_raster_forward(int64_t n, const float* means, const 
     ps.states = reinterpret_cast<unsigned long long*>(ws + L.pair_states);
     ps.failed = &hdr->failed;
     ps.err = device_error_word();
+    ps.limit = kWaitLimit;
     const ListArgs la{hdr, order[kDepthPasses & 1], at(L.offsets), at(L.starts), rect, reach, rows, td.x_bits, cam.tx};
     const nasg_status e = most > kLargePairs
                               ? pair_sort<kLargeThreads, kLargeItems>(la, ps, td, most, keys, vals, ranges, s)
                               : pair_sort<kSmallThreads, kSmallItems>(la, ps, td, most, keys, vals, ranges, s);
     if (e != NASG_OK) return give_up(e, s);
   }
+  if (!set_failed(kBeforeRender)) return give_up(check_launch(), s);
   const uint32_t* list = vals[td.passes & 1];
   auto* ncontrib = at(L.ncontrib);
   const nasg_status e =
@@ -1296,6 +1305,88 @@ extern "C" nasg_status nasg_raster_forward(int64_t n, const float* means, const 
           : launch_chained(n > 0, render_fwd_kernel<1>, unsigned(tiles), TileShape<1>::NT, 0, s, cam, hdr, ranges, list,
                            splat, colours, image, final_t, ncontrib);
   return e == NASG_OK ? e : give_up(e, s);
+}
+
+extern "C" nasg_status nasg_raster_forward(int64_t n, const float* means, const float* scales, const float* quats,
+                                           const float* opacity, const float* colours,
+                                           const nasg_raster_camera* camera, float* image, float* final_t,
+                                           int64_t max_pairs, void* workspace, size_t workspace_bytes,
+                                           int64_t* n_pairs, void* stream) {
+  return forward(kNowhere, n, means, scales, quats, opacity, colours, camera, image, final_t, max_pairs, workspace,
+                 workspace_bytes, n_pairs, stream);
+}
+
+extern "C" nasg_status nasg_probe_raster_failed(int32_t where, int64_t n, const float* means, const float* scales,
+                                                const float* quats, const float* opacity, const float* colours,
+                                                const nasg_raster_camera* camera, float* image, float* final_t,
+                                                int64_t max_pairs, void* workspace, size_t workspace_bytes,
+                                                void* stream) {
+  if (where != kBeforeSorts && where != kBeforeRender) return NASG_ERR_RANGE;
+  return forward(FailAt(where), n, means, scales, quats, opacity, colours, camera, image, final_t, max_pairs, workspace,
+                 workspace_bytes, nullptr, stream);
+}
+
+// ---------------------------------------------------------------------------
+// Diagnostic: sort and scan blocks whose first predecessor never publishes
+// ---------------------------------------------------------------------------
+namespace nasg {
+namespace raster {
+
+constexpr int kProbeBlocks = NASG_PROBE_LOOK_BACK_BLOCKS;  // after block 0; more than a look-back reads at once
+
+struct ProbeStates {
+  unsigned long long sort[kProbeBlocks + 1][sort::kBins], scan[kProbeBlocks + 1];
+};
+static_assert(sizeof(ProbeStates) <= NASG_PROBE_LOOK_BACK_BYTES, "the header's size");
+
+// results[b - 1]: entries that sort block b placed, or -1; results[kProbeBlocks + b - 1]: the scan's count
+// before block b, or -1; results[2 kProbeBlocks]: the `failed` word.
+__global__ void __launch_bounds__(kSmallThreads) look_back_probe_kernel(sort::Pass ps, int first,
+                                                                       unsigned long long* scan, int32_t* results) {
+  extern __shared__ __align__(16) unsigned char sort_smem[];
+  auto& s = *reinterpret_cast<sort::Block<kSmallThreads, kSmallItems>*>(sort_smem);
+  const uint32_t block = blockIdx.x + uint32_t(first);
+  uint32_t key[kSmallItems], val[kSmallItems];
+  for (int i = 0; i < kSmallItems; ++i) key[i] = val[i] = threadIdx.x + uint32_t(i) * kSmallThreads;
+  const int placed = sort::sort_block<kSmallThreads, kSmallItems, false>(s, ps, block, 0u, key, val);
+  if (threadIdx.x < 32) {
+    if (threadIdx.x == 0) sort::st_state(scan + block, (block == 0 ? sort::kAll : sort::kOwn) | sort::tag_bits(ps.tag) | 1u);
+    unsigned long long before = 0;
+    const bool ok = block == 0 || sort::look_back_warp(scan, block, ps.tag, ps.limit, ps.err, &before);
+    if (threadIdx.x == 0 && block > 0) {
+      sort::st_state(scan + block, (ok ? sort::kAll : sort::kGone) | sort::tag_bits(ps.tag) | (before + 1u));
+      results[block - 1] = placed;
+      results[kProbeBlocks + block - 1] = ok ? int32_t(before) : -1;
+    }
+  }
+}
+
+}  // namespace raster
+}  // namespace nasg
+
+extern "C" nasg_status nasg_probe_look_back_timeout(int32_t limit, int32_t first, int32_t* results, void* workspace,
+                                                    size_t workspace_bytes, void* stream) {
+  if (limit < 1 || limit > (1 << 20) || (first != 0 && first != 1)) return NASG_ERR_RANGE;
+  if (!results || !workspace) return NASG_ERR_NULL;
+  if (!aligned(results, 4) || !aligned(workspace, 8)) return NASG_ERR_ALIGN;
+  if (workspace_bytes < NASG_PROBE_LOOK_BACK_BYTES) return NASG_ERR_RANGE;
+  cudaStream_t s = as_stream(stream);
+  auto* states = static_cast<ProbeStates*>(workspace);
+  if (cudaMemsetAsync(states, 0, sizeof(ProbeStates), s) != cudaSuccess ||
+      cudaMemsetAsync(results, 0, (2 * kProbeBlocks + 1) * sizeof(int32_t), s) != cudaSuccess)
+    return check_launch();
+  sort::Pass ps{};
+  ps.states = &states->sort[0][0];
+  ps.failed = reinterpret_cast<uint32_t*>(results + 2 * kProbeBlocks);
+  ps.err = device_error_word();
+  ps.bits = 8;
+  ps.tag = 1;
+  ps.limit = uint32_t(limit);
+  constexpr size_t smem = sizeof(sort::Block<kSmallThreads, kSmallItems>);
+  if (const nasg_status e = ensure_smem_limit(reinterpret_cast<const void*>(look_back_probe_kernel), smem); e != NASG_OK)
+    return e;
+  look_back_probe_kernel<<<unsigned(kProbeBlocks + 1 - first), kSmallThreads, smem, s>>>(ps, first, states->scan, results);
+  return check_launch();
 }
 
 extern "C" nasg_status nasg_raster_backward(int64_t n, const float* colours, const nasg_raster_camera* camera,

@@ -39,9 +39,10 @@ __device__ __forceinline__ bool ready(unsigned long long v, uint32_t tag) {
 }
 
 // Polls a predecessor's state until it is published; a state of kGone when it gave up.
-static __device__ __noinline__ unsigned long long wait_state(const unsigned long long* p, uint32_t tag, int* err) {
+static __device__ __noinline__ unsigned long long wait_state(const unsigned long long* p, uint32_t tag, uint32_t limit,
+                                                            int* err) {
   WaitClock clock(global_ns());
-  for (uint32_t it = 1; it < kWaitLimit; ++it) {
+  for (uint32_t it = 1; it < limit; ++it) {
     const unsigned long long v = ld_state(p);
     if (ready(v, tag)) return v;
     if ((it & 255u) == 0 && clock.over(global_ns(), kWaitNs)) break;
@@ -54,7 +55,7 @@ static __device__ __noinline__ unsigned long long wait_state(const unsigned long
 // predecessors are read at once: walked one by one, the read latency of a few hundred blocks
 // that start together would be the pass's time. False when a wait gave up.
 __device__ __forceinline__ bool look_back(const unsigned long long* states, int stride, int col, uint32_t block,
-                                          uint32_t tag, int* err, unsigned long long* before) {
+                                          uint32_t tag, uint32_t limit, int* err, unsigned long long* before) {
   unsigned long long sum = 0;
   for (int64_t p = int64_t(block) - 1; p >= 0; p -= kWindow) {
     unsigned long long w[kWindow];
@@ -63,7 +64,7 @@ __device__ __forceinline__ bool look_back(const unsigned long long* states, int 
       w[i] = p - i >= 0 ? ld_state(states + (p - i) * stride + col) : (kAll | tag_bits(tag));
 #pragma unroll
     for (int i = 0; i < kWindow; ++i) {
-      if (!ready(w[i], tag)) w[i] = wait_state(states + (p - i) * stride + col, tag, err);
+      if (!ready(w[i], tag)) w[i] = wait_state(states + (p - i) * stride + col, tag, limit, err);
       const unsigned long long flag = w[i] & kGone;
       if (flag == kGone) return false;
       sum += w[i] & kCount;
@@ -79,14 +80,14 @@ __device__ __forceinline__ bool look_back(const unsigned long long* states, int 
 
 // The same for one column, by a whole warp: 32 predecessors at once. Every lane gets the sum.
 __device__ __forceinline__ bool look_back_warp(const unsigned long long* states, uint32_t block, uint32_t tag,
-                                               int* err, unsigned long long* before) {
+                                               uint32_t limit, int* err, unsigned long long* before) {
   const int lane = threadIdx.x & 31;
   unsigned long long sum = 0;
   for (int64_t p = int64_t(block) - 1; p >= 0; p -= 32) {
     unsigned long long v = kAll | tag_bits(tag);
     if (p - lane >= 0) {
       v = ld_state(states + p - lane);
-      if (!ready(v, tag)) v = wait_state(states + p - lane, tag, err);
+      if (!ready(v, tag)) v = wait_state(states + p - lane, tag, limit, err);
     }
     const unsigned long long flag = v & kGone;
     if (__any_sync(0xffffffffu, flag == kGone)) return false;
@@ -152,6 +153,7 @@ struct Pass {
   int* err;
   int shift, bits;
   uint32_t tag;
+  uint32_t limit;              // polls of a wait
 };
 
 // Bound: instructions and the wait for the look-back (a pass over 1e6 depth keys 17 us against
@@ -228,7 +230,7 @@ __device__ __forceinline__ int sort_block(Block<THREADS, ITEMS>& s, const Pass& 
   unsigned long long before = 0;
   bool ok = true;
   if (block > 0 && t < bins) {
-    ok = look_back(ps.states, bins, t, block, ps.tag, ps.err, &before);
+    ok = look_back(ps.states, bins, t, block, ps.tag, ps.limit, ps.err, &before);
     st_state(state, (ok ? kAll : kGone) | tag_bits(ps.tag) | ((before + cnt) & kCount));
   }
   if (t < bins) s.base[t] = digit_base + uint32_t(before) - start;

@@ -70,3 +70,44 @@ def test_forward_waits_blocked_where_the_device_asks_for_it(lib):
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     res = subprocess.run([sys.executable, "-c", BLOCKING.format(root=root)], capture_output=True, text=True, timeout=300)
     assert res.returncode == 0, res.stderr[-2000:]
+
+
+def test_look_back_gives_up(lib):
+    """Blocks whose first predecessor never publishes its counts: every one gives up, says so to those after
+    it, in the failure word and in the device status. With that predecessor they place all their entries."""
+    lib.nasg_device_status()
+    placed, before, failed = lib.nasg_probe_look_back_timeout(1 << 20, first=0)
+    lib.nasg_device_status()
+    assert placed == [1024] * lib.LOOK_BACK_BLOCKS and before == list(range(1, lib.LOOK_BACK_BLOCKS + 1)) and failed == 0
+    placed, before, failed = lib.nasg_probe_look_back_timeout(1024, first=1)
+    assert placed == [-1] * lib.LOOK_BACK_BLOCKS and before == [-1] * lib.LOOK_BACK_BLOCKS and failed == 1
+    with pytest.raises(lib.NasgError) as e:
+        lib.nasg_device_status()
+    assert e.value.status == -6
+    lib.nasg_device_status()
+
+
+# 20 x 12 tiles (one pixel per lane) and 60 x 34 (two); small and large sort blocks
+@pytest.mark.parametrize("where", [1, 2])
+@pytest.mark.parametrize("w,h,n,scale", [(320, 192, 5000, 0.05), (960, 540, 450_000, 0.01)])
+def test_failed_lists_give_an_empty_image(lib, where, w, h, n, scale):
+    import ctypes
+
+    import torch
+    args = _scene(n, 8, scale)
+    r = lib.Raster(n, _camera(lib, w, h), 1 << 25)
+    want, T = r.forward(*args)
+    g = torch.randn((h, w, 3), device="cuda")
+    ref = r.backward(args[4], T, g)
+    assert float(T.min()) < 0.9 and float(ref[1].abs().max()) > 0
+    image, final_t = torch.full((h, w, 3), 7.0, device="cuda"), torch.full((h, w), 7.0, device="cuda")
+    p = [lib._ptr(t) for t in args]
+    lib._check(lib.lib.nasg_probe_raster_failed(where, n, *p, ctypes.byref(r.camera), lib._ptr(image), lib._ptr(final_t),
+                                                r.max_pairs, lib._ptr(r.workspace), r.workspace.numel(), lib._stream(None)),
+               "nasg_probe_raster_failed")
+    assert float(image.abs().max()) == 0.0 and float(final_t.min()) == 1.0 and float(final_t.max()) == 1.0
+    gc, go = r.backward(args[4], final_t, g)
+    assert float(gc.abs().max()) == 0.0 and float(go.abs().max()) == 0.0
+    lib.nasg_device_status()
+    again, _ = r.forward(*args)  # the next forward starts afresh
+    assert torch.equal(again, want)

@@ -40,6 +40,7 @@
 
 #include "nasg_cover.h"
 #include "nasg_host.h"
+#include "nasg_list.h"
 #include "nasg_sort.cuh"
 #include "nasg_vec.cuh"
 
@@ -687,10 +688,10 @@ __global__ void __launch_bounds__(THREADS, THREADS > 256 ? 2 : 4) pair_pass_kern
   write_pairs<THREADS, ITEMS, LAST>(s, ps, cnt, kout, vout, ranges, x_bits, tiles_x);
 }
 
-// The list of a tile, [x, y); empty where a sort gave up.
-__device__ __forceinline__ uint2 tile_range(const Header* hdr, const uint2* __restrict__ ranges, int tile) {
+// The list of a tile; empty where a sort gave up.
+__device__ __forceinline__ TileList list_of(const Header* hdr, const uint2* __restrict__ ranges, int tile) {
   const uint2 r = ranges[tile];
-  return hdr->failed ? make_uint2(0u, 0u) : make_uint2(~r.x, r.y);
+  return hdr->failed ? TileList{0u, 0u} : tile_list(r.x, r.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -745,17 +746,17 @@ __device__ __forceinline__ uint32_t reach_mask(const Splat& p, float x0, float y
   return m;
 }
 
-// Stages primitive vals[j] (where j < end) in slot threadIdx.x and the batch's masks. Each warp
+// Stages primitive list[j] (where `has`) in slot threadIdx.x and the batch's masks. Each warp
 // stages 32 slots and turns their reach masks into one word per sub-tile.
 template <int PX>
-__device__ __forceinline__ void stage_batch(Stage<PX>& st, uint32_t j, uint32_t end, float x0, float y0,
-                                            const uint32_t* __restrict__ vals, const Splat* __restrict__ splat,
+__device__ __forceinline__ void stage_batch(Stage<PX>& st, const uint32_t* __restrict__ list, bool has, uint32_t j, float x0,
+                                            float y0, const Splat* __restrict__ splat,
                                             const float* __restrict__ colours, uint32_t* id_out) {
   using TS = TileShape<PX>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t m = 0;
-  if (j < end) {
-    const uint32_t id = vals[j];
+  if (has) {
+    const uint32_t id = list[j];
     if (id_out) *id_out = id;
     Splat p;
     p.a = splat[id].a;
@@ -827,7 +828,7 @@ __global__ void __launch_bounds__(TileShape<PX>::NT) render_fwd_kernel(
   const int pxi = tx * kTile + (warp & 1) * 8 + (lane & 7);
   const int pyi = ty * kTile + (warp >> 1) * TS::H + (lane >> 3);
   const float px = float(pxi) + 0.5f;
-  const uint2 rg = tile_range(hdr, ranges, tile);
+  const TileList list = list_of(hdr, ranges, tile);
   float py[PX], T[PX], c0[PX], c1[PX], c2[PX];
   uint32_t last[PX];
   bool done[PX], inside[PX];
@@ -841,13 +842,14 @@ __global__ void __launch_bounds__(TileShape<PX>::NT) render_fwd_kernel(
     done[p] = !inside[p];
   }
   bool live = true;  // warp-uniform: some pixel of the warp has not stopped
-  for (uint32_t b = rg.x; b < rg.y; b += TS::NT) {
+  for (ListWalk b(list); b.left > 0; b.next(TS::NT)) {
     bool all = true;
 #pragma unroll
     for (int p = 0; p < PX; ++p) all = all && done[p];
     live = !__all_sync(0xffffffffu, all);
     if (!__syncthreads_or(live)) break;
-    stage_batch<PX>(st, b + threadIdx.x, rg.y, float(tx * kTile), float(ty * kTile), vals, splat, colours, nullptr);
+    stage_batch<PX>(st, vals, threadIdx.x < b.left, b.place + threadIdx.x, float(tx * kTile), float(ty * kTile), splat,
+                    colours, nullptr);
     __syncthreads();
     for (int q = 0; live && q < TS::WORDS; ++q) {
       uint32_t m = st.mask[warp][q];
@@ -869,7 +871,7 @@ __global__ void __launch_bounds__(TileShape<PX>::NT) render_fwd_kernel(
               c1[p] = fmaf(col.y, w, c1[p]);
               c2[p] = fmaf(col.z, w, c2[p]);
               T[p] = test;
-              last[p] = b - rg.x + uint32_t(k) + 1;
+              last[p] = b.place - list.begin + uint32_t(k) + 1;
             }
           }
         }
@@ -907,7 +909,7 @@ __global__ void __launch_bounds__(TileShape<PX>::NT) render_bwd_kernel(
   const int pxi = tx * kTile + (warp & 1) * 8 + (lane & 7);
   const int pyi = ty * kTile + (warp >> 1) * TS::H + (lane >> 3);
   const float px = float(pxi) + 0.5f;
-  const uint2 rg = tile_range(hdr, ranges, tile);
+  const uint32_t* __restrict__ list = vals + list_of(hdr, ranges, tile).begin;
   float py[PX], T[PX], g0[PX], g1[PX], g2[PX];
   float after[PX];  // sum over later contributions of (c . g) alpha T
   uint32_t last[PX];
@@ -937,8 +939,8 @@ __global__ void __launch_bounds__(TileShape<PX>::NT) render_bwd_kernel(
     const uint32_t hi = n - seen;                            // exclusive end (relative)
     const uint32_t lo = hi > uint32_t(TS::NT) ? hi - TS::NT : 0u;
     uint32_t id = 0;
-    stage_batch<PX>(st, rg.x + lo + threadIdx.x, rg.x + hi, float(tx * kTile), float(ty * kTile), vals, splat, colours,
-                    &id);
+    stage_batch<PX>(st, list, lo + threadIdx.x < hi, lo + threadIdx.x, float(tx * kTile), float(ty * kTile), splat,
+                    colours, &id);
 #pragma unroll
     for (int w = 0; w < TS::W; ++w) s_grad[w][threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();

@@ -526,7 +526,8 @@ nasg_status nasg_raster_forward(int64_t n, const float* means, const float* scal
  *   dC/dc_i = alpha_i T_i,  dC/dalpha_i = c_i T_i - (sum_{later j} c_j alpha_j T_j)/(1 - alpha_i),
  *   dalpha_i/dsigma_i = rho_i where alpha_i < 0.99.
  * final_t: the forward's output; g_image device [height][width][3] f32. Sums over
- * pixels use float atomics (the summation order is not fixed).
+ * pixels use float atomics (the summation order is not fixed). After a forward that was
+ * refused with NASG_ERR_CAPACITY both are zero.
  */
 nasg_status nasg_raster_backward(int64_t n, const float* colours, const nasg_raster_camera* camera,
                                  const float* final_t, const float* g_image, float* g_colours, float* g_opacity,

@@ -1083,11 +1083,14 @@ struct HostWords {
   }
 };
 
-// For a forward that ends without its image: waits for the stream, so that nothing of the call is left
-// running. The caller may then free or reuse the workspace (n_pairs is reported so that it can make a
-// larger one), and no late store reaches the thread's words under a later call's number.
-inline nasg_status give_up(nasg_status why, cudaStream_t s) {
+// For a forward that ends without its image: the pixels' counts are cleared (they are an earlier image's,
+// and a backward would take them for places in lists that are not there), and the stream is waited for, so
+// that nothing of the call is left running. The caller may then free or reuse the workspace (n_pairs is
+// reported so that it can make a larger one), and no late store reaches the thread's words under a later
+// call's number.
+inline nasg_status give_up(nasg_status why, uint32_t* ncontrib, int64_t pixels, cudaStream_t s) {
   const BesideCaptures beside;
+  cudaMemsetAsync(ncontrib, 0, size_t(pixels) * sizeof(uint32_t), s);
   cudaStreamSynchronize(s);
   cudaGetLastError();  // `why` stands; its CUDA error, if it has one, is recorded
   return why;
@@ -1249,20 +1252,22 @@ static nasg_status forward(FailAt fail, int64_t n, const float* means, const flo
   const TileDigits td = tile_digits(cam.tx, cam.ty);
 
   if (cudaMemsetAsync(ws + L.header, 0, L.head_end - L.header, s) != cudaSuccess) return check_launch();
+  auto* ncontrib = at(L.ncontrib);
+  auto refuse = [&](nasg_status why) { return give_up(why, ncontrib, pixels, s); };
   auto set_failed = [&](FailAt where) {
     return fail != where || cudaMemsetAsync(&hdr->failed, 1, 1, s) == cudaSuccess;
   };
-  if (!set_failed(kBeforeSorts)) return give_up(check_launch(), s);
+  if (!set_failed(kBeforeSorts)) return refuse(check_launch());
   unsigned long long total64 = 0;
   if (n > 0) {
     static thread_local HostWords host;
-    if (!host.ready()) return give_up(check_launch(), s);
+    if (!host.ready()) return refuse(check_launch());
     const unsigned long long call = ++host.calls;
     ProjectArgs pa{n, means, scales, quats, opacity, cam, td, splat, rows, rect, reach, dkeys[0], hdr, host.words, call};
     const int64_t blocks = (n + kBlock - 1) / kBlock;
     const int64_t most = int64_t(sm_count()) * 4;
     project_kernel<<<unsigned(blocks < most ? blocks : most), kBlock, 0, s>>>(pa);
-    if (const nasg_status e = check_launch(); e != NASG_OK) return give_up(e, s);
+    if (const nasg_status e = check_launch(); e != NASG_OK) return refuse(e);
     sort::Pass ps{};
     ps.states = reinterpret_cast<unsigned long long*>(ws + L.depth_states);
     ps.failed = &hdr->failed;
@@ -1271,19 +1276,19 @@ static nasg_status forward(FailAt fail, int64_t n, const float* means, const flo
     nasg_status e = n > kLargeDepth
                               ? depth_sort<kLargeThreads, kLargeItems>(ps, hdr, dkeys, order, uint32_t(n), s)
                               : depth_sort<kSmallThreads, kSmallItems>(ps, hdr, dkeys, order, uint32_t(n), s);
-    if (e != NASG_OK) return give_up(e, s);
+    if (e != NASG_OK) return refuse(e);
     constexpr int64_t kChunk = kBlock * kScanItems;
     e = launch_chained(true, offsets_kernel, unsigned((n + kChunk - 1) / kChunk), kBlock, 0, s, hdr,
                        hdr->tickets + kDepthPasses, ps.err, (unsigned long long)(max_pairs),
                        reinterpret_cast<ulonglong2*>(ws + L.pair_states),
                        reinterpret_cast<unsigned long long*>(ws + L.scan_states), order[kDepthPasses & 1], reach,
                        at(L.offsets), at(L.starts));
-    if (e != NASG_OK) return give_up(e, s);
+    if (e != NASG_OK) return refuse(e);
     // the host waits for the projection's total while the GPU sorts by depth
-    if (!wait_total(host.words, call, s, &total64)) return give_up(NASG_ERR_CUDA, s);
+    if (!wait_total(host.words, call, s, &total64)) return refuse(NASG_ERR_CUDA);
   }
   if (n_pairs) *n_pairs = int64_t(total64);
-  if (int64_t(total64) > max_pairs) return give_up(NASG_ERR_CAPACITY, s);
+  if (int64_t(total64) > max_pairs) return refuse(NASG_ERR_CAPACITY);
   if (total64 > 0) {
     const int64_t most = int64_t(total64);  // at least the pairs listed
     sort::Pass ps{};
@@ -1295,18 +1300,17 @@ static nasg_status forward(FailAt fail, int64_t n, const float* means, const flo
     const nasg_status e = most > kLargePairs
                               ? pair_sort<kLargeThreads, kLargeItems>(la, ps, td, most, keys, vals, ranges, s)
                               : pair_sort<kSmallThreads, kSmallItems>(la, ps, td, most, keys, vals, ranges, s);
-    if (e != NASG_OK) return give_up(e, s);
+    if (e != NASG_OK) return refuse(e);
   }
-  if (!set_failed(kBeforeRender)) return give_up(check_launch(), s);
+  if (!set_failed(kBeforeRender)) return refuse(check_launch());
   const uint32_t* list = vals[td.passes & 1];
-  auto* ncontrib = at(L.ncontrib);
   const nasg_status e =
       two_pixels(tiles, 8)
           ? launch_chained(n > 0, render_fwd_kernel<2>, unsigned(tiles), TileShape<2>::NT, 0, s, cam, hdr, ranges, list,
                            splat, colours, image, final_t, ncontrib)
           : launch_chained(n > 0, render_fwd_kernel<1>, unsigned(tiles), TileShape<1>::NT, 0, s, cam, hdr, ranges, list,
                            splat, colours, image, final_t, ncontrib);
-  return e == NASG_OK ? e : give_up(e, s);
+  return e == NASG_OK ? e : refuse(e);
 }
 
 extern "C" nasg_status nasg_raster_forward(int64_t n, const float* means, const float* scales, const float* quats,

@@ -111,3 +111,21 @@ def test_failed_lists_give_an_empty_image(lib, where, w, h, n, scale):
     lib.nasg_device_status()
     again, _ = r.forward(*args)  # the next forward starts afresh
     assert torch.equal(again, want)
+
+
+# room for the first image's pairs (at most 4 and 64 tiles each), not for every primitive in all 12 and 1200 tiles
+@pytest.mark.parametrize("w,h,room", [(64, 48, 8000), (640, 480, 128_000)])
+def test_backward_after_a_refused_forward(lib, w, h, room):
+    """The refused forward leaves its workspace the counts of the image before it and no lists: gradients zero."""
+    import torch
+    n = 2000
+    args = _scene(n, 9, 0.03)
+    r = lib.Raster(n, _camera(lib, w, h), room)
+    _, T = r.forward(*args)
+    g = torch.randn((h, w, 3), device="cuda")
+    assert float(r.backward(args[4], T, g)[1].abs().max()) > 0
+    with pytest.raises(lib.NasgError) as e:
+        r.forward(args[0], args[1] * 1e4, *args[2:])
+    assert e.value.status == -7
+    gc, go = r.backward(args[4], T, g)
+    assert float(gc.abs().max()) == 0.0 and float(go.abs().max()) == 0.0

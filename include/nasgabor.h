@@ -345,9 +345,9 @@ size_t nasgabor_batched_workspace_bytes(int32_t n_scenes);
 
 /*
  * Validates the scenes (HOST array of n_scenes) and writes their device table
- * and tile ranges (tiles of sub_tiles sub-tiles of I x 256/S primitives, S the
- * lanes per primitive of the scene's L, I = 2 or 3 (by the batch's size) for BF16 and 1
- * for FP32 parameters, 1 <= sub_tiles <= 64)
+ * and tile ranges (direct loads: tiles of sub_tiles sub-tiles of I x 256/S primitives,
+ * S the lanes per primitive of the scene's L, I = 2 for BF16 and 1 for FP32 parameters,
+ * 1 <= sub_tiles <= 64; staged: single sub-tiles, I = 2 or 3 by the batch for BF16)
  * into `workspace` (16-byte aligned, >= nasgabor_batched_workspace_bytes).
  * Synchronises `stream` (not for use inside a stream capture). The buffers the
  * scenes point to are read/written by later runs, not by this call.

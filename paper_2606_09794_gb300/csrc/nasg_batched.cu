@@ -7,12 +7,12 @@
 // scheduling, by a 4-byte counter reset), so a stream capture of it records a
 // CUDA graph that can be replayed. Work items are tiles of k sub-tiles of
 // I x 256/S primitives of one scene (S = lanes per primitive for that scene's L,
-// I = batch_items: a thread evaluates I items of each sub-tile one after the other).
+// I = direct_items: a thread evaluates I items of each sub-tile one after the other).
 // Blocks take tiles round-robin (static) or from an atomic counter (dynamic),
 // look the scene up in the shared-memory copy of the table, and evaluate the
 // tile with the lobe-pair lanes of the single-scene kernels, fetching each
 // lane's next sub-tile item before computing the current one. No thread waits
-// on another block. A staged variant moves each sub-tile's parameter spans,
+// on another block. A staged variant takes single sub-tiles (I = batch_items) and moves each one's parameter spans,
 // means, upstream gradients and diffuse colours into shared memory with bulk
 // copies (span plans for any N), two (BF16) or three (FP32) sub-tiles ahead (one elected producer
 // thread, full/empty mbarriers, every wait bounded), for the scenes whose planes
@@ -29,12 +29,12 @@ namespace nasg {
 struct SceneDev {
   EvalArgs args;       // the scene as the single-scene argument block, read in place from shared
                        // memory by the item arithmetic (no per-thread copy in registers)
-  int64_t tile_begin;  // first global tile of this scene
-  int64_t unit_begin;  // first global sub-tile (tile_begin x sub_tiles)
+  int64_t tile_begin;  // first tile of this scene in the direct kernel
+  int64_t unit_begin;  // first sub-tile of this scene in the staged kernel
   int32_t staged;  // bit 0: parameter spans may be moved by bulk copies (even L >= 4, N L sizeof(T) % 16 == 0,
                    // 16-byte aligned planes); bit 1: the means, upstream gradients and diffuse colours
                    // too (16-byte aligned buffers, moved by span plans)
-  int32_t items;   // items per thread in a sub-tile (I), the same for the whole batch
+  int32_t items;   // items per thread in a staged sub-tile (I), the same for the whole batch
 };
 
 constexpr int kMaxScenes = NASG_MAX_SCENES;
@@ -45,7 +45,7 @@ struct BatchArgs {
   uint32_t* counter;  // dynamic scheduling
   int32_t n_scenes;
   int32_t sub_tiles;  // k
-  int64_t total_tiles;
+  int64_t total_tiles;  // of the direct kernel
   int32_t dynamic;
   int* dev_err;
 };
@@ -114,20 +114,26 @@ __device__ __forceinline__ void eval_scene_item(const EvalArgs& a, const RawItem
 // then as given (the table is internal; each record holds its scene's own buffers).
 inline int lobe_class(int32_t L) { return L == 4 ? 0 : (L == 8 ? 1 : (L == 16 ? 2 : 3)); }
 
-// Items per thread in a sub-tile. BF16: three, so that the wait for a stage, the producer's turn
-// and the scene's lookup are shared by three items, while that leaves each block of two per SM
-// at least eight sub-tiles; else two (a last round of large sub-tiles leaves more blocks idle). 16
-// scenes of 1.05e7 primitives: 1311 us unrolled with two items and three stages, 1252 us not
-// unrolled, 1242 us with two stages, 1217 us with three items; 6 scenes of up to 3e5: 111, 107, 105,
-// 104 us; 3 scenes of 75 000 primitives: 10.4 us with two items, 12.4 us with three.
+// Items per thread in a sub-tile of the direct kernel, where they only set the size of a tile: with as many
+// as the staged kernel takes (three for large BF16 batches), four sub-tiles made 256 scenes of 2000 to 7000 x 8
+// lobes 2 to 10 % slower (98.4 -> 105.9 us, 277.4 -> 282.2 us).
+template <typename T>
+constexpr int direct_items() { return sizeof(T) == 2 ? 2 : 1; }
+
+// Items per thread in a sub-tile of the staged kernel. BF16: three, so that the wait for a stage, the
+// producer's turn and the scene's lookup are shared by three items, while that leaves each block of two per
+// SM at least eight sub-tiles; else two (a last round of large sub-tiles leaves more blocks idle). 16 scenes of
+// 1.05e7 primitives: 1242 us with two items, 1208 us with three; 6 scenes of up to 3e5: 105 and 104 us; 3
+// scenes of 75 000 primitives in all: 10.4 and 12.4 us.
 static int batch_items(const nasg_scene* scenes, int32_t n_scenes, int32_t param_dtype) {
   if (param_dtype != NASG_DTYPE_BF16) return unit_items<float>();
   const int most = unit_items<__nv_bfloat16>();
   const int64_t enough = int64_t(sm_count()) * 2 * 8 * 256 * most;  // lanes
   int64_t lanes = 0;
-  for (int j = 0; j < n_scenes && lanes < enough; ++j)
-    if (scenes[j].n > 0 && scenes[j].n_lobes >= 1 && scenes[j].n_lobes <= NASG_MAX_LOBES)
-      lanes += std::min<int64_t>(scenes[j].n, enough) << slice_log2(scenes[j].n_lobes);
+  for (int j = 0; j < n_scenes; ++j) {
+    if (scenes[j].n <= 0 || scenes[j].n_lobes < 1 || scenes[j].n_lobes > NASG_MAX_LOBES) continue;
+    lanes += std::min<int64_t>(scenes[j].n, int64_t(1) << 40) << slice_log2(scenes[j].n_lobes);
+  }
   return lanes >= enough ? most : most - 1;
 }
 
@@ -162,7 +168,7 @@ __global__ void __launch_bounds__(256, 2) batched_kernel(const BatchArgs b) {
     const int tp = 256 >> sc.slice_log2;
     const int local = threadIdx.x >> sc.slice_log2;
     const int l0 = 2 * (threadIdx.x & ((1 << sc.slice_log2) - 1));
-    const int sub = b.sub_tiles * sd[lo].items;  // sub-items of tp primitives in the tile
+    const int sub = b.sub_tiles * direct_items<T>();  // sub-items of tp primitives in the tile
     const int64_t base = (tile - sd[lo].tile_begin) * int64_t(tp) * sub;
     RawItem<T, P> cur, nxt;
     fetch_scene_item<T, P>(sc, base + local, l0, true, cur);
@@ -205,7 +211,7 @@ constexpr uint32_t kUnitEnd = 0xffffffffu;
 // Shared-memory metadata of one stage, written by the producer with the unit.
 struct StageMeta {
   uint32_t unit;     // global sub-tile index, kUnitEnd past the last
-  int32_t scene;     // scene index, -1 for an empty unit
+  int32_t scene;     // scene index, -1 past the last
   int32_t staged;    // bit 0: parameter spans in the stage; bit 1: means and upstream gradients too
   int32_t count;     // primitives in the unit
   int64_t p0;        // first primitive of the unit in its scene
@@ -224,20 +230,10 @@ __host__ __device__ inline uint32_t batch_stage_bytes() {
 // copies were started (the stage then completes when their bytes have landed).
 // A block's units increase, so the scene is found by advancing `sc_i` (the
 // previous unit's scene); a scene's units are its sub-tiles in order, from
-// tile_begin x sub_tiles, so the unit's first primitive needs no division.
+// unit_begin, so the unit's first primitive needs no division.
 template <typename T, int P>
 __device__ __forceinline__ bool issue_unit(const BatchArgs& b, const SceneDev* sd, uint32_t unit, int& sc_i,
                                            StageMeta* meta, unsigned char* st, uint64_t* bar) {
-  const int64_t total_units = b.total_tiles * b.sub_tiles;
-  if (int64_t(unit) >= total_units) {
-    meta->unit = kUnitEnd;
-    meta->scene = -1;
-    meta->staged = 0;
-    meta->count = 0;
-    meta->p0 = 0;
-    mbar_arrive(bar);
-    return false;
-  }
   const int64_t u = int64_t(unit);
   while (sc_i + 1 < b.n_scenes && sd[sc_i + 1].unit_begin <= u) ++sc_i;
   const EvalArgs& sc = sd[sc_i].args;
@@ -246,13 +242,22 @@ __device__ __forceinline__ bool issue_unit(const BatchArgs& b, const SceneDev* s
   const uint32_t L = uint32_t(sc.n_lobes);
   const int64_t tp = int64_t(256 >> sc.slice_log2) * sd[sc_i].items;
   const int64_t p0 = (u - sd[sc_i].unit_begin) * tp;
+  if (p0 >= n) {  // past the last scene's units
+    meta->unit = kUnitEnd;
+    meta->scene = -1;
+    meta->staged = 0;
+    meta->count = 0;
+    meta->p0 = 0;
+    mbar_arrive(bar);
+    return false;
+  }
   const int64_t count = n - p0 < tp ? n - p0 : tp;
   meta->unit = unit;
-  meta->scene = count > 0 ? sc_i : -1;
-  meta->count = count > 0 ? int32_t(count) : 0;
+  meta->scene = sc_i;
+  meta->count = int32_t(count);
   meta->p0 = p0;
-  const uint32_t bytes = count > 0 ? uint32_t(count) * L * uint32_t(sizeof(T)) : 0u;
-  const bool stage_p = count > 0 && (staged & 1) && (bytes % 16u) == 0u;
+  const uint32_t bytes = uint32_t(count) * L * uint32_t(sizeof(T));
+  const bool stage_p = (staged & 1) && (bytes % 16u) == 0u;
   const bool stage_m = stage_p && (staged & 2);
   meta->staged = (stage_p ? 1 : 0) | (stage_m ? 2 : 0);
   if (!stage_p) {
@@ -462,7 +467,7 @@ extern "C" nasg_status nasgabor_batched_prepare(const nasg_scene* scenes, int32_
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
     return lobe_class(scenes[x].n_lobes) < lobe_class(scenes[y].n_lobes);
   });
-  int64_t tiles = 0, prims = 0, lobes = 0;
+  int64_t tiles = 0, units = 0, prims = 0, lobes = 0;
   const int items = batch_items(scenes, n_scenes, modes->param_dtype);
   bool pair_path = true;
   for (int j = 0; j < n_scenes; ++j) {
@@ -512,14 +517,17 @@ extern "C" nasg_status nasgabor_batched_prepare(const nasg_scene* scenes, int32_
                    ? 1 | (aligned(s.means, 16) && aligned(s.g_rgb, 16) && aligned(s.c0, 16) ? 2 : 0)
                    : 0;
     d.tile_begin = tiles;
-    d.unit_begin = tiles * sub_tiles;
+    d.unit_begin = units;
     d.items = items;
-    const int64_t tile_prims = int64_t(256 >> a.slice_log2) * items * sub_tiles;
+    const int64_t row = 256 >> a.slice_log2, unit_prims = row * items;
+    const int64_t tile_prims =
+        row * (modes->param_dtype == NASG_DTYPE_BF16 ? direct_items<__nv_bfloat16>() : direct_items<float>()) * sub_tiles;
     tiles += (s.n + tile_prims - 1) / tile_prims;
+    units += (s.n + unit_prims - 1) / unit_prims;
     prims += s.n;
     lobes += s.n * s.n_lobes;
   }
-  if (tiles >= (int64_t(1) << 32)) return NASG_ERR_RANGE;
+  if (tiles >= (int64_t(1) << 32) || units >= (int64_t(1) << 32) - (int64_t(1) << 20)) return NASG_ERR_RANGE;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   cudaStream_t st = as_stream(stream);
   if (cudaMemsetAsync(ws, 0, kBatchHeader, st) != cudaSuccess ||
@@ -561,8 +569,8 @@ static nasg_status launch_batched_k(const BatchArgs& b, int blocks_per_sm, bool 
       fit = 1;
     const int per_sm = blocks_per_sm > 0 && blocks_per_sm < fit ? blocks_per_sm : fit;
     int64_t grid = int64_t(sm_count()) * per_sm;
-    const int64_t units = b.total_tiles * b.sub_tiles;
-    if (grid > units) grid = units;
+    const int64_t most = b.total_tiles * b.sub_tiles;  // at least the sub-tiles
+    if (grid > most) grid = most;
     if (grid < 1) return NASG_OK;
     k<<<unsigned(grid), kStagedThreads, smem, s>>>(b);
     return check_launch();

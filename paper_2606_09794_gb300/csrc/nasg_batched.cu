@@ -124,17 +124,21 @@ constexpr int direct_items() { return sizeof(T) == 2 ? 2 : 1; }
 // producer's turn and the scene's lookup are shared by three items, while that leaves each block of two per
 // SM at least eight sub-tiles; else two (a last round of large sub-tiles leaves more blocks idle). 16 scenes of
 // 1.05e7 primitives: 1242 us with two items, 1208 us with three; 6 scenes of up to 3e5: 105 and 104 us; 3
-// scenes of 75 000 primitives in all: 10.4 and 12.4 us.
+// scenes of 75 000 primitives in all: 10.4 and 12.4 us. Two as well where scenes of odd lobe counts, which
+// find their items in no stage and load each in turn, are most of the work: 64 scenes of 8000 primitives and 3
+// to 11 lobes 184 and 190 us.
 static int batch_items(const nasg_scene* scenes, int32_t n_scenes, int32_t param_dtype) {
   if (param_dtype != NASG_DTYPE_BF16) return unit_items<float>();
   const int most = unit_items<__nv_bfloat16>();
   const int64_t enough = int64_t(sm_count()) * 2 * 8 * 256 * most;  // lanes
-  int64_t lanes = 0;
+  int64_t lanes = 0, odd = 0;
   for (int j = 0; j < n_scenes; ++j) {
     if (scenes[j].n <= 0 || scenes[j].n_lobes < 1 || scenes[j].n_lobes > NASG_MAX_LOBES) continue;
-    lanes += std::min<int64_t>(scenes[j].n, int64_t(1) << 40) << slice_log2(scenes[j].n_lobes);
+    const int64_t l = std::min<int64_t>(scenes[j].n, int64_t(1) << 40) << slice_log2(scenes[j].n_lobes);
+    lanes += l;
+    if (scenes[j].n_lobes % 2 != 0) odd += l;
   }
-  return lanes >= enough ? most : most - 1;
+  return lanes >= enough && 2 * odd <= lanes ? most : most - 1;
 }
 
 // FLAGS: kFlagsDefault (raw activations, approximate normalisation) or

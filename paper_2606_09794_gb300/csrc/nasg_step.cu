@@ -250,7 +250,7 @@ __device__ __forceinline__ void step_phase2(const StepArgs& s, IDX i, int l0, co
 // How a step kernel moves master, m and v. kScalar: element loads in phase two (odd L, unaligned
 // buffers). kPairs: each lane copies its own lobe pairs to shared memory (8 bytes, through L1).
 // kQuads: neighbouring lanes share their copies, 16 bytes each, past L1 (L a multiple of
-// four, 16-byte aligned planes).
+// four but 12, 16-byte aligned planes; see step_kernel).
 enum StepMove { kScalar, kPairs, kQuads };
 
 // Shared memory of the step kernel: per thread, P gradient pairs and, but for kScalar, the P
@@ -287,13 +287,22 @@ __device__ __forceinline__ void copy_quads(float2* slot, const float* planes, ID
     if (p + 1 < P || !odd) cp_async16(dst + p * 256, planes + off);
 }
 
+// Copies the P planes of the lane's own two lobes. off: the first of them in plane 0.
+template <int P, typename IDX>
+__device__ __forceinline__ void copy_pairs(float2* slot, const float* planes, IDX off, IDX NL) {
+  float2* dst = slot + threadIdx.x;
+#pragma unroll
+  for (int p = 0; p < P; ++p, off += NL) cp_async8(dst + p * 256, planes + off);
+}
+
 // Bound: HBM, and how many bytes the SM has in flight (16 warps, 128 registers, issue 31 %). Copies
 // of 8 bytes land through L1, whose lines are what is left of 80 KB x 2 of shared memory: with
 // 100 KB per block (a master copy one item ahead) the step took 1.4 times as long. 16-byte copies
 // past L1 have no such limit and are half as many: 6e6-primitive shell, 45 % visible, 8 lobes,
 // 1102 -> 1024 us per camera (5.8 TB/s); every primitive 2221 -> 2034 us (6.5 TB/s). On top of them
 // a master copy (1043 us) or the list's entry (1053 us) one item ahead, or streaming stores of m
-// and v (1082 us), gained nothing.
+// and v (1082 us), gained nothing. 16-byte copies gain 4 to 10 % at L = 4, 8, 16, 20, 24, 28 and 32 (4e6 lobes,
+// every primitive), and lose 8 % at L = 12 (236 / 255 us), whose rows of 48 bytes stay with the 8-byte ones.
 template <int FRAME, typename IDX, int MOVE, bool LOSS>
 __global__ void __launch_bounds__(256, 2) step_kernel(const StepArgs s) {
   constexpr int P = FrameTraits<FRAME>::P;
@@ -319,6 +328,7 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepArgs s) {
     float2* varr = marr + kSlots;
     float2* tarr = varr + kSlots;
     const IDX lq = IDX(l0 & ~3);  // the quad's first lobe
+    const bool gaps = L == 4 && a.idx;
     const bool has_lobes = IDX(l0) < L;
     // block-uniform loop: every lane of a warp reaches the shuffles in phase one
     for (IDX t0 = IDX(blockIdx.x) * blockDim.x; t0 < total; t0 += stride) {
@@ -326,13 +336,25 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepArgs s) {
       IDX i = 0;
       const bool ok = step_prim(a, total, t0 + threadIdx.x, i);
       cur.ok = ok;
+      // A list's entry of four lobes is half a sector. Where the warp's entries are not neighbours, 8-byte copies
+      // through L1: of 10^6 primitives 45 % at random, ascending, 232 -> 228 us, 70 % 250 -> 238 us (8-byte copies
+      // alone 224 and 236 us, but 117 us instead of 113 us for every other run of 40)
+      const bool run = !gaps || __all_sync(0xffffffffu, i == __shfl_sync(0xffffffffu, i, 0) + IDX((threadIdx.x & 31) >> 1));
       __syncwarp();  // the warp has read its slots
-      if (ok && has_lobes) copy_quads<P>(tarr, master, i * L + lq, NL);
+      if (ok && has_lobes) {
+        if (run) copy_quads<P>(tarr, master, i * L + lq, NL);
+        else copy_pairs<P>(tarr, master, i * L + IDX(l0), NL);
+      }
       cp_async_commit();
       if (ok) {
         if (has_lobes) {
-          copy_quads<P>(marr, s.m, i * L + lq, NL);
-          copy_quads<P>(varr, s.v, i * L + lq, NL);
+          if (run) {
+            copy_quads<P>(marr, s.m, i * L + lq, NL);
+            copy_quads<P>(varr, s.v, i * L + lq, NL);
+          } else {
+            copy_pairs<P>(marr, s.m, i * L + IDX(l0), NL);
+            copy_pairs<P>(varr, s.v, i * L + IDX(l0), NL);
+          }
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -672,7 +694,7 @@ extern "C" nasg_status nasgabor_fused_step(const nasg_desc* desc, const nasg_tra
   const bool even = desc->n_lobes % 2 == 0 && aligned(st->master, 8) && aligned(st->m, 8) && aligned(st->v, 8) &&
                     (!st->params_bf16 || aligned(st->params_bf16, 4));
   const int64_t NL = desc->n * desc->n_lobes;
-  const bool quads = even && desc->n_lobes % 4 == 0 && aligned(st->master, 16) && aligned(st->m, 16) && aligned(st->v, 16);
+  const bool quads = even && desc->n_lobes % 4 == 0 && desc->n_lobes != 12 && aligned(st->master, 16) && aligned(st->m, 16) && aligned(st->v, 16);
   const StepMove move = quads ? kQuads : (even ? kPairs : kScalar);
   const int64_t lim = int64_t(1) << 31;
   const bool idx32 = NL * nasg_lobe_planes(desc->frame_mode) < lim && 3 * desc->n < lim &&

@@ -411,7 +411,10 @@ extern "C" nasg_status nasgabor_fit_step(const nasg_desc* desc, const nasg_train
   a.exact = desc->norm_mode == NASG_NORM_EXACT;
   a.partials = static_cast<float*>(workspace);
   // the fitting workload's shape (16 student, 4 teacher lobes) runs a fixed-count instance
-  const bool shared = n_dirs <= kFitSharedDirs;
+  // Shared directions gain 1 to 5 % but in the run-time instance at many lobes, which the added registers cost
+  // more: 1e5 primitives, 64 directions, 16 and 8 lobes 750 -> 758 us, 16 and 16 918 -> 928 us; 16 and 4 (the fixed
+  // instance) 652 -> 622 us, 8 and 4 385 -> 382 us, 4 and 2 205 us either way, exact normalisation 707 -> 697 us.
+  const bool shared = n_dirs <= kFitSharedDirs && (a.exact || ls < 16 || teacher_lobes == 4);
   auto pick = [&](auto sh) {
     constexpr bool SH = decltype(sh)::value;
     return a.exact ? fit_kernel<true, 0, 0, SH>

@@ -484,7 +484,8 @@ typedef struct nasg_raster_camera {
 } nasg_raster_camera;
 
 /* Device workspace bytes for n primitives, a width x height image and room for
- * max_pairs (tile, primitive) pairs; 0 if out of range. */
+ * max_pairs (tile, primitive) pairs; 0 if out of range. About 96 bytes per primitive, 16 per
+ * pair and 4 per pixel (1e6 primitives at 1920 x 1080 with 1.4e7 pairs: 332 MB). */
 size_t nasg_raster_workspace_bytes(int64_t n, int32_t width, int32_t height, int64_t max_pairs);
 
 /*

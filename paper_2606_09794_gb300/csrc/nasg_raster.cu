@@ -224,11 +224,10 @@ struct HostTotal {
 
 // Programmatic dependent launch: a kernel of the forward's chain lets the next one start when its
 // blocks have only their results to write, and reads or writes nothing before its predecessor
-// has finished, so that a launch's latency passes meanwhile (640 x 360 preview of 2e4 primitives
-// 137 -> 116 us, with the total left in page-locked words by the projection itself instead of a copy
-// and an event, and the pair states cleared by the offset scan). Allowed at the start of the blocks
+// has finished, so that a launch's latency passes meanwhile: the ten launches of a 640 x 360 preview of
+// 2e4 primitives take 124 us one by one and 112 us chained. Allowed at the start of the blocks
 // instead, the next pass's blocks crowd onto the SMs that the running pass leaves free (two of
-// 512 threads on one, none on another): 8e5 primitives at 320 x 180 288 -> 337 us.
+// 512 threads on one, none on another): 8e5 primitives at 320 x 180 337 us instead of 288 us.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -338,10 +337,11 @@ __device__ __forceinline__ uint32_t project_one(const ProjectArgs& a, int64_t i,
   return count;
 }
 
-// Projection of every primitive and, beside it, all the counts that the sorts start from: one
-// pass in place of histogram launches (1e6 primitives, 1.39e7 pairs of squares: 16 -> 50 us here,
-// against 195 us of histogram launches and 149 us of scans before). The grid is a few blocks per SM, so that a block's shared
-// counts go to global memory once for many primitives.
+// Projection of every primitive and, beside it, all the counts that the sorts start from, which
+// would otherwise take a launch over the keys for each pass (1e6 primitives, 1.4e7 pairs of squares: 58 us
+// here, of them 16 us the projection; as launches of their own the counts took 98 us). Bound: the atomics on the
+// block's shared counts. The grid is a few blocks per SM, so that those go to global memory once for many
+// primitives.
 __global__ void __launch_bounds__(kBlock) project_kernel(const ProjectArgs a) {
   __shared__ Counts counts;
   __shared__ unsigned long long s_pairs;
@@ -573,8 +573,8 @@ struct ListArgs {
   int tiles_x;
 };
 
-// First pass of the pair sort, 146 us of emission and 211 us of its radix pass before, 106 us now
-// (1e6 primitives at 1080p). A block's pairs are places [base, base + THREADS ITEMS) of the depth
+// First pass of the pair sort (1e6 primitives at 1080p: 111 us; issue 39 % active, the leading stalls
+// barriers, loads of the primitives' rows and shared-memory traffic). A block's pairs are places [base, base + THREADS ITEMS) of the depth
 // order's list: it finds the primitives that hold them in `starts` and writes their tiles into
 // shared memory itself, so the list never goes through memory unsorted. A thread lists a
 // primitive of up to kAlone tiles alone; a warp shares the rows of a larger one.
@@ -698,14 +698,11 @@ __device__ __forceinline__ TileList list_of(const Header* hdr, const uint2* __re
 // Tile rendering
 // ---------------------------------------------------------------------------
 
-// Bound: issue (73-77 % of the slots in both passes); DRAM is idle. With one pixel per
-// lane in 16 x 2 strips, every warp walked the tile's whole list, most of it primitives whose
-// footprint square meets the tile and whose ellipse misses the strip. Masks per 8 x 8 or 8 x 4
-// sub-tile cost one thread about 40 operations per (tile, primitive) and cut the walked
-// (warp, primitive) visits; two pixels per lane share the staged reads, the terms in x
-// and, backward, the shuffles; one atomic per tile instead of per warp. 1e6 primitives at
-// 1920 x 1080, forward and backward with sorts: 2533 -> 1661 us; 3e5 at 1280 x 720 in
-// a training frame: 1376 -> 964 us.
+// Bound: issue (78 % of the slots in both passes at 1e6 primitives and 1920 x 1080, 258 us forward and 405 us
+// backward; FMA pipe 49 and 42 % busy, DRAM idle at 2 %). Most primitives whose footprint square meets a tile
+// miss most of its pixels: masks per 8 x 8 or 8 x 4 sub-tile cost one thread about 40 operations per
+// (tile, primitive) and save the warps the visits. Two pixels per lane share the staged reads, the terms in
+// x and, backward, the shuffles; a tile adds each of its sums once.
 //
 // Pixels of a tile among its warps. PX = 2: four warps, one 8 x 8 quadrant each, a lane
 // holding pixels (x, y) and (x, y + 4); PX = 1: eight warps of 8 x 4 pixels, one per lane.
@@ -784,8 +781,8 @@ __device__ __forceinline__ void stage_batch(Stage<PX>& st, const uint32_t* __res
 // alpha of staged primitive k at the lane's pixels; 0 when below 1/255. Every operation is
 // explicitly rounded so that the forward and the backward kernels take the same decisions on
 // the same inputs. Two pixels go through packed FP32x2 operations, each component rounded as the
-// scalar one, so both layouts give the same bits (1080p, 1e6 primitives: forward 271 -> 261 us,
-// backward 432 -> 415 us; the operands are staged twice to be had without moves).
+// scalar one, so both layouts give the same bits (1080p, 1e6 primitives: forward 261 us, with
+// scalar operations 271 us, backward 415 and 432 us; the operands are staged twice to be had without moves).
 template <int PX>
 __device__ __forceinline__ void pixel_alpha(const Stage<PX>& st, int k, float px, const float* py, float* alpha,
                                             float* rho) {
@@ -970,7 +967,7 @@ __global__ void __launch_bounds__(TileShape<PX>::NT) render_bwd_kernel(
           if (al[p] > 0.f) {
             // 1/(1 - alpha), 1 - alpha in [0.01, 1]: the approximation and one Newton step, against 64
             // bits no further off than the division (g_opacity 1.01e-6 either way at 1080p, without the
-            // pixels whose stop differs) and a third of its instructions: 489 -> 432 us
+            // pixels whose stop differs) and a third of its instructions (1080p: 432 us, divided 489 us)
             const float om = 1.f - al[p], r0 = rcpa(om);
             const float inv = fmaf(r0, fmaf(-om, r0, 1.f), r0);
             const float Tb = T[p] * inv;  // transmittance in front of this contribution

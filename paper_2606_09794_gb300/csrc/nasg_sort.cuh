@@ -156,8 +156,8 @@ struct Pass {
   uint32_t limit;              // polls of a wait
 };
 
-// Bound: instructions and the wait for the look-back (a pass over 1e6 depth keys 17 us against
-// 37 us for histogram, three scan launches and scatter; over the pairs of a 1080p frame 69 us).
+// Bound: instructions and the wait for the look-back (a pass over 1e6 depth keys 17 us, as histogram, three
+// scan launches and scatter 37 us; over the pairs of a 1080p frame 72 us, issue 56 % active, ALU 64 %).
 // Sorts the block's entries (thread's item i at place warp * 32 * ITEMS + 32 i + lane of the
 // block's input; kNone is dropped) by one digit, stable, into s.key / s.val, and finds where
 // each digit's run goes. Returns the number of entries, or a negative number when a wait gave up.
@@ -174,7 +174,7 @@ __device__ __forceinline__ int sort_block(Block<THREADS, ITEMS>& s, const Pass& 
   __syncthreads();
   // lanes of the warp with the same digit: by match.any, whose time grows with the number of
   // different digits in the warp (MATCH: passes whose neighbours share digits, the lists' columns and
-  // the depths' upper bits: 133 -> 109 us and 16 -> 12 us at 1080p), or bit by bit (the others: 69
+  // the depths' upper bits: 109 us, bit by bit 133, and 12 us, 16, at 1080p), or bit by bit (the others: 69
   // against 78 us and 17 against 20 us). The first of them adds their number to the warp's count, in
   // the items' order.
 #pragma unroll

@@ -167,10 +167,12 @@ template <bool BWD>
 static nasg_status launch_sh(int degree, const ShArgs& a, cudaStream_t s) {
   constexpr int kBlock = 256;
   const unsigned grid = grid_for(a.n, kBlock);
-  // Coefficients that do not fit L2 (129 MB) beside the rest are streamed: degree 3 of 1e6 (192 MB)
-  // 39.0 -> 34.5 us, degree 2 of 1e6 (108 MB) 24.3 -> 20.7 us; smaller ones may be in L2 and should
-  // stay there for the next pass (degree 3 of 1e5, 19 MB, again and again: 5.3 us, streamed 8.2 us). The
-  // backward, which writes as much as it reads, is slower streamed (67 -> 72 us).
+  // Coefficients that do not fit L2 (129 MB) beside the rest are streamed. Passes over the same inputs again and
+  // again, read as usual / streamed: forward alone at degree 3, 1e6 primitives (192 MB) 39.4 / 34.7 us, 525 000
+  // (101 MB) 21.2 / 20.8 us, degree 2, 1.1e6 (119 MB) 25.6 / 21.6 us; forward and its backward, which then finds less
+  // of them in L2, 109.1 / 103.4, 62.6 / 58.0 and 72.1 / 68.8 us. After a flush of L2 the pair is within 3 % either
+  // way. Smaller coefficients may be in L2 and should stay there for the next pass (degree 3 of 1e5, 19 MB: 5.3 us,
+  // streamed 8.2 us). The backward, which writes as much as it reads, is slower streamed (67, 72 us).
   const bool stream = a.n * int64_t(12) * (degree + 1) * (degree + 1) >= int64_t(100) * 1000 * 1000;
   switch (degree) {
 #define NASG_SH_CASE(D)                                                   \

@@ -882,7 +882,10 @@ nasg_status launch_eval(const nasg_desc* desc, EvalArgs a, cudaStream_t s) {
   a.dev_err = device_error_word();
   a.slice_log2 = slice_log2(desc->n_lobes);
   a.slice = 1 << a.slice_log2;
-  a.width = eval_width(desc->n_lobes, a.slice);
+  // host memory keeps the slices: over the link the groups' stores, whose planes' rows start anywhere in a warp,
+  // lose more than the idle lanes do (4e5 BF16 lobes, slices / groups: L = 5 155 / 183 us, L = 20 141 / 147 us; L = 17
+  // 174 / 167 us, the other lobe counts within 1 %)
+  a.width = a.no_staging ? a.slice : eval_width(desc->n_lobes, a.slice);
   const int es = elem_size(desc->param_dtype);
   const bool even = (desc->n_lobes % 2 == 0) && aligned(a.params, uintptr_t(2 * es)) &&
                     (a.g_params == nullptr || aligned(a.g_params, 8));

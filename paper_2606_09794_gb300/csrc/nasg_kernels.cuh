@@ -35,8 +35,8 @@ struct EvalArgs {
   int32_t n_lobes;
   int32_t slice;        // S = next_pow2(ceil(n_lobes / 2)) lanes per primitive
   int32_t slice_log2;
-  int32_t width;        // lanes per primitive in eval_kernel: S, or ceil(n_lobes / 2) where that
-                        // fits more primitives into a warp (see eval_width)
+  int32_t width;        // lanes per primitive in eval_kernel's groups: ceil(n_lobes / 2) where that
+                        // fits more primitives into a warp than S (see eval_width), else S
   int32_t identity;
   int32_t normalised;
   int32_t exact;        // exact normalisation (implies normalised)
@@ -768,11 +768,24 @@ unsigned persistent_grid(K kernel, int64_t threads, int block) {
 template <int MODE, int FRAME, typename T, typename IDX, bool EVEN>
 nasg_status launch_idx_even(const EvalArgs& a, cudaStream_t s) {
   constexpr int kBlock = kEvalBlock;
-  const bool groups = a.width != a.slice;
-  auto k = groups ? eval_kernel<FRAME, T, IDX, MODE, EVEN, true> : eval_kernel<FRAME, T, IDX, MODE, EVEN, false>;
-  const int64_t per_warp = 32 / a.width;
-  const int64_t threads = (a.n_items + per_warp - 1) / per_warp * 32;
-  k<<<persistent_grid(k, threads, kBlock), kBlock, 0, s>>>(a);
+  auto threads = [&](int64_t width) {
+    const int64_t per_warp = 32 / width;
+    return (a.n_items + per_warp - 1) / per_warp * 32;
+  };
+  // rounds of the persistent grid that the items take
+  auto rounds = [&](auto k, int64_t t) {
+    const int64_t cap = int64_t(sm_count()) * blocks_per_sm(reinterpret_cast<const void*>(k), kBlock, 0) * kBlock;
+    return (t + cap - 1) / cap;
+  };
+  auto slices = eval_kernel<FRAME, T, IDX, MODE, EVEN, false>;
+  auto groups = eval_kernel<FRAME, T, IDX, MODE, EVEN, true>;
+  // groups where they save a round: a round of theirs takes longer (their sums are not butterflies of constant
+  // width), and a call of one round is as long as its slowest warp (backward of 1000 primitives: L = 5 4.5 us with
+  // slices, 5.4 us with groups, L = 9 4.4 / 6.2 us; 9000 listed, L = 9 6.4 / 8.3 us)
+  const bool fewer = a.width != a.slice && rounds(groups, threads(a.width)) < rounds(slices, threads(a.slice));
+  const int64_t t = threads(fewer ? a.width : a.slice);
+  auto k = fewer ? groups : slices;
+  k<<<persistent_grid(k, t, kBlock), kBlock, 0, s>>>(a);
   return check_launch();
 }
 
